@@ -1,6 +1,7 @@
 // kernels.cu -- launch geometry and dtype dispatch of the stencil kernel.
 #include "kernels.hpp"
 #include "box2d_fast.cuh"
+#include "row2d_tb.cuh"
 #include "star3d_tb.cuh"
 
 #include <cmath>
@@ -33,18 +34,36 @@ bool fast_box2d_supported(int r, int depth) {
                           (r == 4 && depth <= 2));
 }
 
+// Radius 2, four levels, on 12800^2 FP32: 825 Gcell-steps/s against 730 with
+// the warp strips of row2d_tb.cuh, which give 16 of their 128 columns to the
+// halo there; every other (R, K) is faster in strips (radius 1: 1763 / 1504 at
+// 8 levels, 1828 / 1289 at 4; radius 2: 730 / 605 at 1, 759 / 670 at 2;
+// radius 3: 481 / 368 at 1, 403 / 404 at 3; radius 4: 321 / 246 at 1,
+// 287 / 239 at 2).
+bool wide_box2d(int r, int depth, int64_t nx, int csize) { return r == 2 && depth == 4 && nx % 4 == 0 && csize == 4; }
+
+bool row2d_supported(int shape, int r, int depth, int csize) {
+    if (depth < 1 || r < 1 || r > 4 || (shape != kBox2D && shape != kStar2D)) return false;
+    // FP64 state takes twice the registers
+    if (csize == 8) return depth <= (r <= 2 ? 4 : 2);
+    if (shape == kBox2D) return fast_box2d_supported(r, depth);
+    return depth <= (r == 1 ? 8 : 4);
+}
+
 namespace {
-template <int R, int K> void box_shape(LaunchShape& ls, int64_t nx, int esize) {
-    using S = BoxShape<R, K>;
-    ls.lx = S::LX;
+// The 2D kernel's geometry; ls.grid.x is the strips until choose_row_split.
+void row_shape(LaunchShape& ls, int shape, int r, int depth, int64_t nx, int csize, int esize) {
+    const int kind = shape == kBox2D ? kRowBox : kRowStar;
+    ls.lx = 32 * row_vx(kind, csize, r, depth);
     ls.ly = 1;
-    ls.tx = S::TX;
+    ls.tx = ls.lx - 2 * row_hxa(r, depth);
     ls.ty = 1;
-    ls.block = dim3(S::NT, 1, 1);
-    ls.smem = esize == 4 ? S::template smem<4>() : S::template smem<2>();
-    ls.grid = dim3((unsigned)((nx + S::TX - 1) / S::TX), 1, 1);
+    ls.ragged = nx % 4 != 0;
+    ls.block = dim3(32 * kRowWarps, 1, 1);
+    ls.smem = (size_t)row_smem(kind, csize, esize, r, depth);
+    ls.grid = dim3((unsigned)((nx + ls.tx - 1) / ls.tx), 1, 1);
     ls.ok = true;
-    ls.fast = kFastBox2D;
+    ls.fast = kFastRow2D;
 }
 
 template <int R, int K> void fast_shape(LaunchShape& ls, int64_t ny, int64_t nx, int esize) {
@@ -61,36 +80,35 @@ template <int R, int K> void fast_shape(LaunchShape& ls, int64_t ny, int64_t nx,
 }
 }  // namespace
 
-LaunchShape stencil_launch_shape(int shape, int r, int depth, int64_t ny, int64_t nx, int csize, int esize) {
+LaunchShape stencil_launch_shape(int shape, int r, int depth, int64_t n0, int64_t ny, int64_t nx, int csize, int esize) {
     LaunchShape ls;
     ls.ok = false;
     ls.fast = 0;
+    ls.ragged = false;
     if (depth < 1) return ls;
-    if (shape == kBox2D && csize == 4 && nx % 4 == 0 && fast_box2d_supported(r, depth) &&
-        !std::getenv("SO2DR_GENERIC_KERNEL")) {
-        switch (r * 16 + depth) {
-            case 17: box_shape<1, 1>(ls, nx, esize); break;
-            case 18: box_shape<1, 2>(ls, nx, esize); break;
-            case 19: box_shape<1, 3>(ls, nx, esize); break;
-            case 20: box_shape<1, 4>(ls, nx, esize); break;
-            case 21: box_shape<1, 5>(ls, nx, esize); break;
-            case 22: box_shape<1, 6>(ls, nx, esize); break;
-            case 23: box_shape<1, 7>(ls, nx, esize); break;
-            case 24: box_shape<1, 8>(ls, nx, esize); break;
-            case 33: box_shape<2, 1>(ls, nx, esize); break;
-            case 34: box_shape<2, 2>(ls, nx, esize); break;
-            case 35: box_shape<2, 3>(ls, nx, esize); break;
-            case 36: box_shape<2, 4>(ls, nx, esize); break;
-            case 49: box_shape<3, 1>(ls, nx, esize); break;
-            case 50: box_shape<3, 2>(ls, nx, esize); break;
-            case 51: box_shape<3, 3>(ls, nx, esize); break;
-            case 65: box_shape<4, 1>(ls, nx, esize); break;
-            case 66: box_shape<4, 2>(ls, nx, esize); break;
-        }
-        if (ls.ok) return ls;
+    const bool fast_ok = n0 <= kMaxFastAxis && ny <= kMaxFastAxis && nx <= kMaxFastAxis &&
+                         !std::getenv("SO2DR_GENERIC_KERNEL");
+    if (fast_ok && shape == kBox2D && wide_box2d(r, depth, nx, csize)) {
+        using S = BoxShape<2, 4>;
+        ls.lx = S::LX;
+        ls.ly = 1;
+        ls.tx = S::TX;
+        ls.ty = 1;
+        ls.block = dim3(S::NT, 1, 1);
+        ls.smem = esize == 4 ? S::template smem<4>() : S::template smem<2>();
+        ls.grid = dim3((unsigned)((nx + S::TX - 1) / S::TX), 1, 1);
+        ls.ok = true;
+        ls.fast = kFastBox2D;
+        return ls;
     }
-    if (shape == kStar3D && csize == 4 && fast_star3d_row_ok(nx, esize) && fast_star3d_supported(r, depth) &&
-        !std::getenv("SO2DR_GENERIC_KERNEL")) {
+    // the 2D kernel takes every other 2D launch of a depth it is built for: on
+    // 16384^2 and 5003 x 6001 grids it was faster than the generic kernel at
+    // every depth, radius and type
+    if (fast_ok && row2d_supported(shape, r, depth, csize)) {
+        row_shape(ls, shape, r, depth, nx, csize, esize);
+        return ls;
+    }
+    if (shape == kStar3D && csize == 4 && fast_star3d_row_ok(nx, esize) && fast_star3d_supported(r, depth) && fast_ok) {
         switch (r * 16 + depth) {
             case 17: fast_shape<1, 1>(ls, ny, nx, esize); break;
             case 18: fast_shape<1, 2>(ls, ny, nx, esize); break;
@@ -132,13 +150,20 @@ LaunchShape stencil_launch_shape(int shape, int r, int depth, int64_t ny, int64_
 int stencil_max_depth(int shape, int r, int csize) {
     int best = 0;
     for (int d = 1; d <= 16; ++d) {
-        LaunchShape ls = stencil_launch_shape(shape, r, d, 1024, 1024, csize, csize);
+        LaunchShape ls = stencil_launch_shape(shape, r, d, 1024, 1024, 1024, csize, csize);
         if (ls.ok) best = d;
     }
     return best;
 }
 
 int stencil_occupancy(int dtype, int shape, int r, int depth, const LaunchShape& ls) {
+    if (ls.fast == kFastRow2D) switch (dtype) {
+        case SO2DR_F64: return occupancy_row2d_f64(shape, r, depth, ls);
+        case SO2DR_F32: return occupancy_row2d_f32(shape, r, depth, ls);
+        case SO2DR_BF16: return occupancy_row2d_bf16(shape, r, depth, ls);
+        case SO2DR_F16: return occupancy_row2d_f16(shape, r, depth, ls);
+        default: return 1;
+    }
     switch (dtype) {
         case SO2DR_F64: return occupancy_stencil_f64(shape, r, depth, ls);
         case SO2DR_F32: return occupancy_stencil_f32(shape, r, depth, ls);
@@ -210,8 +235,53 @@ void choose_work_split(LaunchShape& ls, int64_t nout, int r, int depth, int sms,
     }
 }
 
+void choose_row_split(LaunchShape& ls, int64_t nout, int r, int depth, int csize, int sms, int occ, StencilArgs& a) {
+    const int64_t strips = ls.grid.x;
+    const int64_t slots = (int64_t)kRowWarps * (occ > 0 ? occ : 1), G = slots * (sms > 0 ? sms : 1);
+    // rows a segment streams beyond its own, in units of a row at full depth:
+    // the halo (computed by half of the levels on average), the staging fill
+    // and the start of a CTA
+    const double ovh = 1.0 * r * depth + 8;
+    a.split = 1;
+    a.split2 = 0;
+    a.split_at = nout;
+    // Enough rows: one round of long segments over 65% of the rows, one per
+    // resident warp, then short ones (a quarter of that length)
+    const int64_t m = (strips + G - 1) / G;
+    const int64_t n1 = m * G / strips > 0 ? m * G / strips : 1, at = nout * 65 / 100;
+    const double len1 = (double)at / (double)n1;
+    if (len1 >= 3.0 * ovh) {
+        const double len2 = len1 / 4 > 1.5 * ovh ? len1 / 4 : 1.5 * ovh;
+        a.split = (int)n1;
+        a.split_at = at;
+        a.split2 = (int)((double)(nout - at) / len2 + 1);
+    } else {
+        // Few rows: equal segments.  From wmin units on the warps of an SM
+        // share its arithmetic rate, below it each runs at its own pace.
+        const int64_t wmin = csize == 8 ? 4 : (slots < 12 ? slots : 12);
+        double best = -1;
+        for (int64_t q = 1; q <= 4 * slots; q += q < slots ? 1 : slots) {
+            int64_t n = q * (sms > 0 ? sms : 1) / strips;
+            if (n < 1) n = 1;
+            if (n > nout) n = nout;
+            const int64_t per_sm = (strips * n * slots + G - 1) / G;
+            const int64_t busy = per_sm <= slots ? (per_sm > wmin ? per_sm : wmin) : (per_sm + slots - 1) / slots * slots;
+            const double cost = (double)busy * ((double)((nout + n - 1) / n) + ovh);
+            if (best < 0 || cost < best * 0.98) { a.split = (int)n; best = cost; }
+        }
+    }
+    ls.grid.x = (unsigned)((strips * (a.split + a.split2) + kRowWarps - 1) / kRowWarps);
+}
+
 cudaError_t launch_stencil(int dtype, int shape, int r, const StencilArgs& a, const LaunchShape& ls,
                            cudaStream_t s) {
+    if (ls.fast == kFastRow2D) switch (dtype) {
+        case SO2DR_F64: return launch_row2d_f64(shape, r, a, ls, s);
+        case SO2DR_F32: return launch_row2d_f32(shape, r, a, ls, s);
+        case SO2DR_BF16: return launch_row2d_bf16(shape, r, a, ls, s);
+        case SO2DR_F16: return launch_row2d_f16(shape, r, a, ls, s);
+        default: return cudaErrorInvalidValue;
+    }
     switch (dtype) {
         case SO2DR_F64: return launch_stencil_f64(shape, r, a, ls, s);
         case SO2DR_F32: return launch_stencil_f32(shape, r, a, ls, s);

@@ -15,10 +15,16 @@ struct LaunchShape {
     size_t smem;
     int lx, ly, tx, ty;
     bool ok;
-    int fast;    // 0 generic kernel, kFastStar3D (star3d_tb.cuh), kFastBox2D (box2d_fast.cuh)
+    int fast;    // 0 generic kernel, kFastStar3D (star3d_tb.cuh), kFastRow2D (row2d_tb.cuh),
+                 // kFastBox2D (box2d_fast.cuh)
+    bool ragged; // rows are not whole 4-element vectors: the kernels' element-wise staging
 };
 
-constexpr int kFastStar3D = 1, kFastBox2D = 2;
+constexpr int kFastStar3D = 1, kFastRow2D = 2, kFastBox2D = 3;
+
+// Axes the register-streaming kernels index with 32-bit integers end here;
+// longer ones run on the generic kernel.
+constexpr int64_t kMaxFastAxis = (int64_t)1 << 30;
 
 // (R, K) pairs the register-streaming 3D star kernel is instantiated for.
 bool fast_star3d_supported(int r, int depth);
@@ -33,11 +39,18 @@ bool fast_star3d_row_ok(int64_t nx, int esize);
 cudaError_t encode_plane_map(CUtensorMap* map, int esize, const void* base, int64_t nx, int64_t ny, int64_t cap,
                              int box_x, int box_rows);
 
-// (R, K) pairs the register-streaming 2D box kernel is instantiated for.
+// (R, K) pairs of 2D box stencils within which the planner picks its depth.
 bool fast_box2d_supported(int r, int depth);
 
+// Whether the CTA-wide 2D box kernel takes a launch: aligned rows and the one
+// (R, K) at which it is the faster one.
+bool wide_box2d(int r, int depth, int64_t nx, int csize);
+
+// (R, K) pairs the 2D kernel is instantiated for (shape kBox2D or kStar2D).
+bool row2d_supported(int shape, int r, int depth, int csize);
+
 // csize: compute-type bytes; esize: storage-type bytes.
-LaunchShape stencil_launch_shape(int shape, int r, int depth, int64_t ny, int64_t nx, int csize, int esize);
+LaunchShape stencil_launch_shape(int shape, int r, int depth, int64_t n0, int64_t ny, int64_t nx, int csize, int esize);
 
 // Largest fused depth the stencil kernel supports for this geometry.
 int stencil_max_depth(int shape, int r, int csize);
@@ -54,8 +67,8 @@ int stencil_occupancy(int dtype, int shape, int r, int depth, const LaunchShape&
 // share_sm: the occ resident CTAs of an SM share its throughput, so the time
 // goes with the CTAs the busiest SM receives times the planes each streams
 // (the 3D star kernel, issue-bound); otherwise they run side by side and the
-// time goes with the waves of sms * occ CTAs (the 2D box kernel, whose second
-// resident CTA hides the first one's latency).
+// time goes with the waves of sms * occ CTAs (the CTA-wide 2D box kernel,
+// whose second resident CTA hides the first one's latency).
 int choose_segments(int64_t tiles, int64_t nout, int r, int depth, int sms, int occ, bool share_sm);
 
 // Work split of a 3D star kernel launch (ls.grid is tiles in x by tiles in
@@ -68,6 +81,21 @@ int choose_segments(int64_t tiles, int64_t nout, int r, int depth, int sms, int 
 // units of at most 384 planes.  SO2DR_WORK_SPLIT=grid|rounds pins the choice
 // (waves: the grid split with segments counted in waves of resident CTAs).
 void choose_work_split(LaunchShape& ls, int64_t nout, int r, int depth, int sms, int occ, int* split);
+
+// Work split of a 2D kernel launch: sets a.split, a.split2 and a.split_at
+// (axis-0 segments per strip) and ls.grid.x (the strips before the call, the
+// CTAs after it).
+void choose_row_split(LaunchShape& ls, int64_t nout, int r, int depth, int csize, int sms, int occ, StencilArgs& a);
+
+// 2D kernel (row2d_tb.cuh), one translation unit per storage type.
+int occupancy_row2d_f64(int shape, int r, int depth, const LaunchShape& ls);
+int occupancy_row2d_f32(int shape, int r, int depth, const LaunchShape& ls);
+int occupancy_row2d_bf16(int shape, int r, int depth, const LaunchShape& ls);
+int occupancy_row2d_f16(int shape, int r, int depth, const LaunchShape& ls);
+cudaError_t launch_row2d_f64(int shape, int r, const StencilArgs& a, const LaunchShape& ls, cudaStream_t s);
+cudaError_t launch_row2d_f32(int shape, int r, const StencilArgs& a, const LaunchShape& ls, cudaStream_t s);
+cudaError_t launch_row2d_bf16(int shape, int r, const StencilArgs& a, const LaunchShape& ls, cudaStream_t s);
+cudaError_t launch_row2d_f16(int shape, int r, const StencilArgs& a, const LaunchShape& ls, cudaStream_t s);
 
 // Per-dtype instantiations (one translation unit each).
 int occupancy_stencil_f64(int shape, int r, int depth, const LaunchShape& ls);

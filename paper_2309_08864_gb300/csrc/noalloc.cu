@@ -154,7 +154,7 @@ extern "C" int so2dr_run_device_noalloc(int ndim, const int64_t* dims, int radiu
     for (int64_t j = 0; j < L; ++j) {
         const int depth = (j < nfull) ? k_on : (int)res;
         void* dst = ((L - 1 - j) % 2 == 0) ? d_out : scratch;
-        LaunchShape ls = stencil_launch_shape(shape, radius, depth, ny, nx, csize, (int)esize);
+        LaunchShape ls = stencil_launch_shape(shape, radius, depth, n0, ny, nx, csize, (int)esize);
         if (!ls.ok) return set_error(SO2DR_E_UNSUPPORTED, "fused depth too large for the stencil kernel");
         ls.grid.z = 1;
         StencilArgs a;
@@ -162,7 +162,8 @@ extern "C" int so2dr_run_device_noalloc(int ndim, const int64_t* dims, int radiu
         if (ls.fast) {
             int occ = stencil_occupancy(dtype, shape, radius, depth, ls);
             if (ls.fast == kFastStar3D) choose_work_split(ls, n0, radius, depth, sms, occ, &a.split);
-            else ls.grid.z = (unsigned)choose_segments((int64_t)ls.grid.x * ls.grid.y, n0, radius, depth, sms, occ, false);
+            else if (ls.fast == kFastBox2D) ls.grid.z = (unsigned)choose_segments((int64_t)ls.grid.x * ls.grid.y, n0, radius, depth, sms, occ, false);
+            else choose_row_split(ls, n0, radius, depth, csize, sms, occ, a);
         }
         a.in = src;
         a.in_cap = n0;

@@ -164,7 +164,7 @@ int enqueue_stencil(so2dr_plan_s* P, const RunList& rl, const Op& op, cudaStream
     const so2dr_op_t& o = op.pub;
     int shape = shape_of(p);
     int csize = p.dtype == SO2DR_F64 ? 8 : 4;
-    LaunchShape ls = stencil_launch_shape(shape, p.r, o.depth, p.ny, p.nx, csize, (int)p.elem_bytes);
+    LaunchShape ls = stencil_launch_shape(shape, p.r, o.depth, p.n0, p.ny, p.nx, csize, (int)p.elem_bytes);
     ls.grid.z = 1;
     if (!ls.ok) return set_error(SO2DR_E_UNSUPPORTED, "fused depth too large for the stencil kernel");
     // host-side argument checks (the kernel trusts them)
@@ -230,9 +230,11 @@ int enqueue_stencil(so2dr_plan_s* P, const RunList& rl, const Op& op, cudaStream
             if (a.split && o.stream >= 0 && o.stream < kNumStreams)
                 a.work_ctr = reinterpret_cast<unsigned*>(P->arena + rl.arena_bytes - kAlign + kWorkCtrOff +
                                                          8 * o.stream);
-        } else {
+        } else if (ls.fast == kFastBox2D) {
             int64_t tiles = (int64_t)ls.grid.x * ls.grid.y;
             ls.grid.z = (unsigned)choose_segments(tiles, o.dst_hi - o.dst_lo, p.r, o.depth, P->sm_count, occ, false);
+        } else {
+            choose_row_split(ls, o.dst_hi - o.dst_lo, p.r, o.depth, csize, P->sm_count, occ, a);
         }
     } else {
         // generic kernel: axis-0 segments too, so that a launch of few tiles

@@ -55,6 +55,10 @@ struct StencilArgs {
     // the tiles x n (tile, segment) units in rounds (the last round's units
     // cut shorter along axis 0)
     int split;
+    // 2D kernel: `split` segments per strip over the first split_at output
+    // rows, split2 shorter ones over the rest
+    int split2;
+    int64_t split_at;
     // round split: {next piece, finished CTAs}, zero at launch; the CTAs take
     // pieces in order from this counter (null: CTA c takes pieces c, c + G, ...)
     // and the last CTA to finish zeroes both for the next launch on the stream

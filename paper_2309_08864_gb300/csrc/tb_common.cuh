@@ -1,5 +1,5 @@
 // tb_common.cuh -- device helpers shared by the register-streaming
-// temporal-blocking kernels (star3d_tb.cuh, box2d_fast.cuh): storage <-> FP32
+// temporal-blocking kernels (star3d_tb.cuh, row2d_tb.cuh): storage <-> FP32
 // vector conversions, cp.async staging, and the mbarrier / TMA primitives of
 // sm_103a written as inline PTX.
 #pragma once
@@ -25,6 +25,13 @@ __device__ __forceinline__ void cp_async16(void* sdst, const void* gsrc, bool va
     unsigned sa = (unsigned)__cvta_generic_to_shared(sdst);
     int n = valid ? 16 : 0;
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sa), "l"(gsrc), "r"(n));
+}
+// one 4- or 8-byte element, aligned to its size; zero-filled when !valid
+template <typename T> __device__ __forceinline__ void cp_async_elem(T* sdst, const T* gsrc, bool valid) {
+    static_assert(sizeof(T) == 4 || sizeof(T) == 8, "cp.async copies 4, 8 or 16 bytes");
+    unsigned sa = (unsigned)__cvta_generic_to_shared(sdst);
+    int n = valid ? (int)sizeof(T) : 0;
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;\n" ::"r"(sa), "l"(gsrc), "n"(sizeof(T)), "r"(n));
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
 template <int N> __device__ __forceinline__ void cp_async_wait_group() {
