@@ -18,7 +18,8 @@ LIB = os.path.join(HERE, "libso2dr.so")
 BUILD_DIR = os.path.join(HERE, "_build")
 
 CU_SOURCES = ["run.cu", "kernels.cu", "tma_map.cu", "adjoint.cu", "noalloc.cu", "tune.cu", "stencil_f64.cu", "stencil_f32.cu",
-              "stencil_bf16.cu", "stencil_f16.cu", "row2d_f64.cu", "row2d_f32.cu", "row2d_bf16.cu", "row2d_f16.cu"]
+              "stencil_bf16.cu", "stencil_f16.cu", "star3d_f32.cu", "star3d_bf16.cu", "star3d_f16.cu",
+              "star3d_ragged_f32.cu", "star3d_ragged_bf16.cu", "star3d_ragged_f16.cu", "row2d_f64.cu", "row2d_f32.cu", "row2d_bf16.cu", "row2d_f16.cu"]
 CXX_SOURCES = ["plan.cpp"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

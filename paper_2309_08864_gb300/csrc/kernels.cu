@@ -75,6 +75,8 @@ template <int R, int K> void fast_shape(LaunchShape& ls, int64_t ny, int64_t nx,
     ls.block = dim3(S::NT, 1, 1);
     ls.smem = esize == 4 ? S::template smem<4>() : S::template smem<2>();
     ls.grid = dim3((unsigned)((nx + S::TX - 1) / S::TX), (unsigned)((ny + S::TY - 1) / S::TY), 1);
+    ls.ragged = !fast_star3d_row_ok(nx, esize);
+    if (ls.ragged) ls.smem += S::ragged_bytes;
     ls.ok = ls.grid.y <= 65535;
     ls.fast = kFastStar3D;
 }
@@ -108,7 +110,7 @@ LaunchShape stencil_launch_shape(int shape, int r, int depth, int64_t n0, int64_
         row_shape(ls, shape, r, depth, nx, csize, esize);
         return ls;
     }
-    if (shape == kStar3D && csize == 4 && fast_star3d_row_ok(nx, esize) && fast_star3d_supported(r, depth) && fast_ok) {
+    if (shape == kStar3D && csize == 4 && fast_star3d_supported(r, depth) && fast_ok) {
         switch (r * 16 + depth) {
             case 17: fast_shape<1, 1>(ls, ny, nx, esize); break;
             case 18: fast_shape<1, 2>(ls, ny, nx, esize); break;
@@ -157,6 +159,12 @@ int stencil_max_depth(int shape, int r, int csize) {
 }
 
 int stencil_occupancy(int dtype, int shape, int r, int depth, const LaunchShape& ls) {
+    if (ls.fast == kFastStar3D) switch (dtype) {
+        case SO2DR_F32: return ls.ragged ? occupancy_star3d_ragged_f32(r, depth, ls) : occupancy_star3d_f32(r, depth, ls);
+        case SO2DR_BF16: return ls.ragged ? occupancy_star3d_ragged_bf16(r, depth, ls) : occupancy_star3d_bf16(r, depth, ls);
+        case SO2DR_F16: return ls.ragged ? occupancy_star3d_ragged_f16(r, depth, ls) : occupancy_star3d_f16(r, depth, ls);
+        default: return 1;
+    }
     if (ls.fast == kFastRow2D) switch (dtype) {
         case SO2DR_F64: return occupancy_row2d_f64(shape, r, depth, ls);
         case SO2DR_F32: return occupancy_row2d_f32(shape, r, depth, ls);
@@ -275,6 +283,12 @@ void choose_row_split(LaunchShape& ls, int64_t nout, int r, int depth, int csize
 
 cudaError_t launch_stencil(int dtype, int shape, int r, const StencilArgs& a, const LaunchShape& ls,
                            cudaStream_t s) {
+    if (ls.fast == kFastStar3D) switch (dtype) {
+        case SO2DR_F32: return ls.ragged ? launch_star3d_ragged_f32(r, a, ls, s) : launch_star3d_f32(r, a, ls, s);
+        case SO2DR_BF16: return ls.ragged ? launch_star3d_ragged_bf16(r, a, ls, s) : launch_star3d_bf16(r, a, ls, s);
+        case SO2DR_F16: return ls.ragged ? launch_star3d_ragged_f16(r, a, ls, s) : launch_star3d_f16(r, a, ls, s);
+        default: return cudaErrorInvalidValue;
+    }
     if (ls.fast == kFastRow2D) switch (dtype) {
         case SO2DR_F64: return launch_row2d_f64(shape, r, a, ls, s);
         case SO2DR_F32: return launch_row2d_f32(shape, r, a, ls, s);

@@ -87,6 +87,21 @@ void choose_work_split(LaunchShape& ls, int64_t nout, int r, int depth, int sms,
 // CTAs after it).
 void choose_row_split(LaunchShape& ls, int64_t nout, int r, int depth, int csize, int sms, int occ, StencilArgs& a);
 
+// 3D star kernel (star3d_tb.cuh), a translation unit per storage type and
+// kind of rows.
+int occupancy_star3d_f32(int r, int depth, const LaunchShape& ls);
+cudaError_t launch_star3d_f32(int r, const StencilArgs& a, const LaunchShape& ls, cudaStream_t s);
+int occupancy_star3d_bf16(int r, int depth, const LaunchShape& ls);
+cudaError_t launch_star3d_bf16(int r, const StencilArgs& a, const LaunchShape& ls, cudaStream_t s);
+int occupancy_star3d_f16(int r, int depth, const LaunchShape& ls);
+cudaError_t launch_star3d_f16(int r, const StencilArgs& a, const LaunchShape& ls, cudaStream_t s);
+int occupancy_star3d_ragged_f32(int r, int depth, const LaunchShape& ls);
+cudaError_t launch_star3d_ragged_f32(int r, const StencilArgs& a, const LaunchShape& ls, cudaStream_t s);
+int occupancy_star3d_ragged_bf16(int r, int depth, const LaunchShape& ls);
+cudaError_t launch_star3d_ragged_bf16(int r, const StencilArgs& a, const LaunchShape& ls, cudaStream_t s);
+int occupancy_star3d_ragged_f16(int r, int depth, const LaunchShape& ls);
+cudaError_t launch_star3d_ragged_f16(int r, const StencilArgs& a, const LaunchShape& ls, cudaStream_t s);
+
 // 2D kernel (row2d_tb.cuh), one translation unit per storage type.
 int occupancy_row2d_f64(int shape, int r, int depth, const LaunchShape& ls);
 int occupancy_row2d_f32(int shape, int r, int depth, const LaunchShape& ls);

@@ -1,0 +1,7 @@
+// star3d_bf16.cu -- 3D star temporal-blocking kernels for bf16 storage.
+#include <cstring>
+#define STORAGE_T __nv_bfloat16
+#define STAGE_RAGGED 0
+#define STAR_LAUNCH_FN launch_star3d_bf16
+#define STAR_OCC_FN occupancy_star3d_bf16
+#include "star3d_inst.inc"

@@ -85,6 +85,15 @@ template <int R, int K> struct StarShape {
     template <int ES> static constexpr int smem() {
         return kBarBytes + NI * in_slot_bytes<ES>() + (K - 1) * NB * lev_bytes;
     }
+    static constexpr int ragged_bytes = NW * LX * 4;    // output rows of a launch on ragged rows
+};
+
+// How a launch stages its input planes.
+enum StageMode : int {
+    kStageTma = 0,     // TMA boxes of the input buffer (rows are whole 16-byte units)
+    kStageHost = 1,    // TMA boxes, and planes of the mapped host grid (zero-copy input)
+    kStageRagged = 2,  // element by element (any row length): a tensor map cannot describe
+                       // rows that are no multiple of 16 bytes
 };
 
 // How a warp treats the fixed boundary in a phase.
@@ -94,12 +103,13 @@ enum BndMode : int {
     kBndCells = 2,    // boundary rows or fixed planes: per-cell masks
 };
 
-template <typename T, int R, int K, bool ZC>
+template <typename T, int R, int K, int STG>
 struct StarTB {
     using S = StarShape<R, K>;
     static constexpr int VY = S::VY, NW = S::NW, LX = S::LX, LYT = S::LYT, ROWS = S::ROWS, NI = S::NI,
-                         PD = S::PD, NB = S::NB, W2 = 2 * R, ES = (int)sizeof(T), LXB = S::template lxb<ES>(),
-                         SLOT = S::template in_slot_bytes<ES>();
+                         PD = S::PD, NB = S::NB, W2 = 2 * R, ES = (int)sizeof(T);
+    static constexpr bool ZC = STG == kStageHost, RAG = STG == kStageRagged;
+    static constexpr int LXB = RAG ? LX : S::template lxb<ES>(), SLOT = S::template in_slot_bytes<ES>();
     static constexpr unsigned kAll = (1u << (4 * VY)) - 1u;
     static constexpr int kWorkOff = 64;  // work-split constants, behind the mbarriers
     static_assert(NI * 8 <= kWorkOff && kWorkOff + 8 * 4 <= S::kBarBytes, "barrier block layout");
@@ -108,6 +118,7 @@ struct StarTB {
     const CUtensorMap* tmap;
     uint32_t bar0, sin0;  // shared addresses: mbarrier 0, input slot 0
     const T* sin;         // [NI] slots of [ROWS][LXB] staged input
+    float* sout;          // ragged rows: [NW][LX] output rows on their way out
     float* slev;          // [K-1][NB][ROWS][LX] completed planes of levels 0..K-2
     int lane, warp, my_row, col0;
     int n0, ny, nx, xs, ys, gx0, bx0;
@@ -190,6 +201,38 @@ struct StarTB {
             if (gy < ny && gx < nx)
                 *reinterpret_cast<uint4*>(dst + (int64_t)gy * nx + gx) =
                     *reinterpret_cast<const uint4*>(sb + (gy - ys + R) * LXB + (gx - bx0));
+        }
+    }
+
+    // all threads: the box of phase q element by element into its slot, zeros
+    // outside the grid.  4-byte elements, and pairs of 16-bit ones in rows of
+    // even length, go as 4-byte cp.async copies; 16-bit elements of odd rows
+    // (below cp.async's granularity) through registers.
+    __device__ __forceinline__ void stage_ragged(int q) {
+        const int z = za + q;
+        if (z >= zb) return;
+        const int slot = (int)((a.in_slot0 + (int64_t)(z - (int)a.in_lo)) % a.in_cap);
+        const T* base = static_cast<const T*>(a.in) + (int64_t)slot * plane;
+        T* sb = const_cast<T*>(sin) + ((gb + q) % NI) * (SLOT / ES);
+        if (ES == 4 || nx % 2 == 0) {
+            constexpr int PE = 4 / ES, CW = LX / PE;  // elements per copy, copies per row
+            const int c = (threadIdx.x % CW) * PE, gx = xs + c;
+            const bool xok = gx >= 0 && gx < nx;
+#pragma unroll 4
+            for (int row = threadIdx.x / CW; row < ROWS; row += S::NT / CW) {
+                const int gy = ys - R + row;
+                const bool ok = xok && gy >= 0 && gy < ny;
+                cp_async_elem(reinterpret_cast<float*>(sb + row * LXB + c),
+                              reinterpret_cast<const float*>(ok ? base + (int64_t)gy * nx + gx : base), ok);
+            }
+        } else {
+            const int c = threadIdx.x % LX, gx = xs + c;
+            const bool xok = gx >= 0 && gx < nx;
+#pragma unroll 4
+            for (int row = threadIdx.x / LX; row < ROWS; row += S::NT / LX) {
+                const int gy = ys - R + row;
+                sb[row * LXB + c] = xok && gy >= 0 && gy < ny ? base[(int64_t)gy * nx + gx] : T(0.f);
+            }
         }
     }
 
@@ -295,8 +338,26 @@ struct StarTB {
     __device__ __forceinline__ void emit(const float2 (&done)[VY][2], int zt) {
         if (zt < olo || zt >= ohi) return;
         const int lx0 = lane * 4;
-        if (!(lx0 >= S::HXA && lx0 < S::HXA + S::TX && xin)) return;
         T* ob = out + (int64_t)(zt - (int)a.out_lo) * plane;
+        if constexpr (RAG) {
+            // through shared memory, so that a warp's stores are contiguous
+            float* so = sout + warp * LX;
+#pragma unroll
+            for (int y = 0; y < VY; ++y) {
+                const int ty = my_row + y, gy = ys + ty;
+                if (ty < S::HY || ty >= S::HY + S::TY || gy >= ny) continue;  // (the same for every lane)
+                __syncwarp();
+                st4(so + lx0, make_float4(done[y][0].x, done[y][0].y, done[y][1].x, done[y][1].y));
+                __syncwarp();
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int j = lane + 32 * e, gx = xs + j;
+                    if (j >= S::HXA && j < S::HXA + S::TX && gx < nx) store_as<T, float>(ob + (int64_t)gy * nx + gx, so[j]);
+                }
+            }
+            return;
+        }
+        if (!(lx0 >= S::HXA && lx0 < S::HXA + S::TX && xin)) return;
 #pragma unroll
         for (int y = 0; y < VY; ++y) {
             const int ty = my_row + y, gy = ys + ty;
@@ -404,6 +465,15 @@ struct StarTB {
     template <int PH>
     __device__ __forceinline__ bool phase(int p0) {
         const int p = p0 + PH;
+        if constexpr (RAG) {
+            cp_async_wait_group<PD - 1>();  // one group per phase: this phase's has landed
+            __syncthreads();
+            stage_ragged(p + PD);
+            cp_async_commit();
+            phase_levels<PH>(p);
+            if constexpr (PH + 1 < W2) return phase<PH + 1>(p0);
+            return true;
+        }
         const int g = (gb + p) % NI;
         bool late = false;
         bool hp = false;
@@ -442,7 +512,7 @@ struct StarTB {
         ys = y0 - S::HY;
         gx0 = xs + lane * 4;
         xin = gx0 >= 0 && gx0 < nx;  // nx % 4 == 0: a vector is all in or all out
-        bx0 = ES == 4 ? xs : (xs & ~7);  // 16-byte aligned box start
+        bx0 = ES == 4 || RAG ? xs : (xs & ~7);  // 16-byte aligned box start
         col0 = (xs - bx0) + lane * 4;
         inyx = 0;
 #pragma unroll
@@ -461,6 +531,8 @@ struct StarTB {
             const int gy = ys + my_row + y;
             brow |= (gy >= 0 && gy < R) || (gy >= ny - R && gy < ny);
         }
+        // (ragged rows: the ring's right columns may straddle two lanes)
+        if constexpr (RAG) brow |= gx0 < nx && gx0 + 4 > nx - R;
         xl = gx0 == 0;
         xr = gx0 == nx - 4;
         if (__any_sync(0xffffffffu, brow || (xl && xr))) wmode = kBndCells;
@@ -503,7 +575,10 @@ struct StarTB {
         // piece, behind the barrier that ended it)
         if (threadIdx.x == 0) fence_proxy_async_smem();
         for (int q = 0; q < PD; ++q) {
-            if constexpr (ZC) {
+            if constexpr (RAG) {
+                stage_ragged(q);
+                cp_async_commit();
+            } else if constexpr (ZC) {
                 if (host_plane(za + q)) stage_host(q);
                 else if (threadIdx.x == 0) issue(q);
                 cp_async_commit();
@@ -521,6 +596,7 @@ struct StarTB {
         sin = reinterpret_cast<const T*>(smem + S::kBarBytes);
         sin0 = bar0 + S::kBarBytes;
         slev = reinterpret_cast<float*>(smem + S::kBarBytes + NI * SLOT);
+        sout = slev + (K - 1) * NB * ROWS * LX;
         lane = threadIdx.x & 31;
         warp = threadIdx.x >> 5;
         my_row = warp * VY;
@@ -627,7 +703,7 @@ struct StarTB {
             }
             __syncthreads();
         }
-        if constexpr (ZC) cp_async_wait_all();  // no cp.async copy outlives the CTA
+        if constexpr (ZC || RAG) cp_async_wait_all();  // no cp.async copy outlives the CTA
         if (a.split && a.work_ctr && threadIdx.x == 0) {
             // the last CTA to finish (every other one has taken its last
             // piece) zeroes the counter for the next launch on this stream
@@ -641,14 +717,13 @@ struct StarTB {
     }
 };
 
-// ZC: the launch reads some input planes from the mapped host grid (zero-copy
-// input); a separate instantiation, so that the launches of the copy-engine
-// pipeline carry none of its code
-template <typename T, int R, int K, bool ZC = false>
-__global__ void __launch_bounds__(StarShape<R, K>::NT, StarShape<R, K>::MINB)
+// One instantiation per staging mode, so that the launches of the copy-engine
+// pipeline on aligned rows carry none of the others' code
+template <typename T, int R, int K, int STG = kStageTma>
+__global__ void __launch_bounds__(StarShape<R, K>::NT, STG == kStageRagged && R > 2 ? 1 : StarShape<R, K>::MINB)
     star3d_tb_kernel(const StencilArgs a, const __grid_constant__ CUtensorMap tmap) {
     extern __shared__ __align__(1024) unsigned char smem_tb[];
-    StarTB<T, R, K, ZC> k(a, &tmap);
+    StarTB<T, R, K, STG> k(a, &tmap);
     k.run(smem_tb);
 }
 
