@@ -1,6 +1,7 @@
 // kernels.cu -- launch geometry and dtype dispatch of the stencil kernel.
 #include "kernels.hpp"
 #include "box2d_fast.cuh"
+#include "plane_tb.cuh"
 #include "row2d_tb.cuh"
 #include "star3d_tb.cuh"
 
@@ -66,6 +67,36 @@ void row_shape(LaunchShape& ls, int shape, int r, int depth, int64_t nx, int csi
     ls.fast = kFastRow2D;
 }
 
+// The plane kernel's tile: the one that computes the fewest rows of 32 cells
+// over the grid (halos and the grid's last, partial tiles included; a row
+// loaded counts 0.3, a phase's barrier and bookkeeping 12).
+void plane_shape(LaunchShape& ls, int r, int depth, int64_t ny, int64_t nx, int csize) {
+    const int H = r * depth;
+    double best = 0;
+    for (int lx : {32, 64})
+        for (int ly = 2 * H + 4; ly <= kPlaneMaxRows * (kPlaneThreads / lx); ly += 4) {
+            const int tx = lx - 2 * H, ty = ly - 2 * H;
+            const int64_t smem = plane_smem_bytes(r, depth, lx, ly, csize);
+            if (tx <= 0 || smem > kSmemLimit) continue;
+            const int64_t gx = (nx + tx - 1) / tx, gy = (ny + ty - 1) / ty;
+            if (gx > 2147483647 || gy > 65535) continue;
+            double rows = 0.3 * ly;
+            for (int l = 1; l <= depth; ++l) rows += ly - 2 * l * r;
+            const double cost = (double)gx * (double)gy * (rows * (lx / 32) + 12.0);
+            if (ls.ok && cost >= best) continue;
+            best = cost;
+            ls.lx = lx;
+            ls.ly = ly;
+            ls.tx = tx;
+            ls.ty = ty;
+            ls.smem = (size_t)smem;
+            ls.grid = dim3((unsigned)gx, (unsigned)gy, 1);
+            ls.ok = true;
+        }
+    ls.block = dim3(kPlaneThreads, 1, 1);
+    ls.fast = kFastPlane3D;
+}
+
 template <int R, int K> void fast_shape(LaunchShape& ls, int64_t ny, int64_t nx, int esize) {
     using S = StarShape<R, K>;
     ls.lx = S::LX;
@@ -124,6 +155,11 @@ LaunchShape stencil_launch_shape(int shape, int r, int depth, int64_t n0, int64_
             case 66: fast_shape<4, 2>(ls, ny, nx, esize); break;
         }
         if (ls.ok) return ls;
+    }
+    if (fast_ok && ny * nx <= kMaxFastAxis && (shape == kVarcoef3D || (shape == kStar3D && csize == 8))) {
+        plane_shape(ls, r, depth, ny, nx, csize);
+        if (ls.ok) return ls;
+        ls.fast = 0;
     }
     int H = r * depth;
     if (is3d(shape)) {

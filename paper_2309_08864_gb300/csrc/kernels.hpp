@@ -16,11 +16,11 @@ struct LaunchShape {
     int lx, ly, tx, ty;
     bool ok;
     int fast;    // 0 generic kernel, kFastStar3D (star3d_tb.cuh), kFastRow2D (row2d_tb.cuh),
-                 // kFastBox2D (box2d_fast.cuh)
+                 // kFastBox2D (box2d_fast.cuh), kFastPlane3D (plane_tb.cuh)
     bool ragged; // rows are not whole 4-element vectors: the kernels' element-wise staging
 };
 
-constexpr int kFastStar3D = 1, kFastRow2D = 2, kFastBox2D = 3;
+constexpr int kFastStar3D = 1, kFastRow2D = 2, kFastBox2D = 3, kFastPlane3D = 4;
 
 // Axes the register-streaming kernels index with 32-bit integers end here;
 // longer ones run on the generic kernel.

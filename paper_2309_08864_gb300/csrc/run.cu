@@ -219,7 +219,7 @@ int enqueue_stencil(so2dr_plan_s* P, const RunList& rl, const Op& op, cudaStream
         a.cf[k] = (float)p.coeffs[k];
         a.cf2[k] = make_float2(a.cf[k], a.cf[k]);
     }
-    if (ls.fast) {
+    if (ls.fast && ls.fast != kFastPlane3D) {
         // split the work so that the grid fills the SMs evenly
         int& occ = P->occ_cache[1][o.depth];
         if (!occ) occ = stencil_occupancy(p.dtype, shape, p.r, o.depth, ls);
@@ -237,7 +237,7 @@ int enqueue_stencil(so2dr_plan_s* P, const RunList& rl, const Op& op, cudaStream
             choose_row_split(ls, o.dst_hi - o.dst_lo, p.r, o.depth, csize, P->sm_count, occ, a);
         }
     } else {
-        // generic kernel: axis-0 segments too, so that a launch of few tiles
+        // generic and plane kernels: axis-0 segments too, so that a launch of few tiles
         // (a narrow 2D grid) still spreads over the SMs (one CTA per SM
         // counted; its shared memory varies with the tile)
         int64_t tiles = (int64_t)ls.grid.x * ls.grid.y;
