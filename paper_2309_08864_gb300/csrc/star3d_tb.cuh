@@ -16,9 +16,12 @@
 //    the box reads zeros where it leaves the grid;
 //  * every fused level keeps 2R partial sums per cell in registers: when the
 //    level below produces plane z', it is added into the targets z'-R..z'+R
-//    (the in-plane terms at z') and target z'-R is complete.  The register
-//    slot of a target is fixed by its plane index modulo 2R and the plane
-//    loop is unrolled 2R times, so the ring never moves data;
+//    (the in-plane terms at z') and target z'-R is complete.  The sums never
+//    move data: at radius 1 the plane loop is unrolled twice and a target's
+//    register slot is fixed; at larger radii every sum takes the next lower
+//    slot as its last product of the plane is added (the FMA's destination),
+//    and the loop is not unrolled, which keeps it inside the instruction
+//    cache;
 //  * levels are pipelined across planes: level L consumes what level L-1
 //    completed in the previous phase, so one barrier per plane suffices.  A
 //    thread's own cells of that plane stay in its registers (levels run from
@@ -35,9 +38,8 @@
 //    flight, select per cell on a slower path;
 //  * a phase runs one body per boundary mode (no boundary cell, ring columns,
 //    per-cell masks); for radius 1 the phases in which every level is active
-//    run straight-line bodies without per-level tests, for larger radii (2R
-//    phases of longer bodies) a uniform per-level test keeps the code inside
-//    the instruction cache.
+//    run straight-line bodies without per-level tests, for larger radii a
+//    uniform per-level test (no straight-line copies: measured the same).
 // The valid area shrinks by R per level in y and x: the compute-area
 // adjustment of Algorithm 1 applied inside a launch.
 //
@@ -74,6 +76,13 @@ template <int R, int K> struct StarShape {
     static constexpr int NI = (R == 4 && K == 1) ? 6 : 4;
     static constexpr int PD = NI - 1;                   // planes loaded ahead
     static constexpr int NB = 2;                        // plane slots per intermediate level
+    // planes per turn of the plane loop: radius 1 is unrolled 2R = 2 times
+    // (fixed register slots; the moving ones spill at four levels: 1489 ->
+    // 1084 Gcell-steps/s on 1024^3); 2R = 4 to 8 such bodies leave the
+    // instruction cache (768^3 in core, unrolled against not: radius 4 376 /
+    // 461 at one level, 110 / 245 at two, radius 3 485 / 515 and 329 / 357,
+    // 1024^3 radius 2 770 / 859 at two)
+    static constexpr int UNR = R == 1 ? 2 : 1;
     static constexpr int MINB = K == 1 ? 2 : 1;         // CTAs per SM the registers are sized for
     // staged columns: 16-bit boxes start on an 8-element boundary (16 bytes),
     // so they carry 8 spare columns and the tile starts 0 or 4 columns in
@@ -254,8 +263,7 @@ struct StarTB {
         }
     }
 
-    // One arrival at level L whose target phase is PHL = (zp - za) mod 2R:
-    // v holds my cells of the arriving plane, `rows` its shared-memory copy
+    // One arrival at level L (PHL: the arriving plane's phase mod UNR): v holds my cells of the arriving plane, `rows` its shared-memory copy
     // (tile row t at row t + R, my first column at element col).  Masks
     // mz[t] (t = 0..R, kBndCells only) belong to targets zp - R + t.
     template <int L, int PHL, int MODE, typename ST>
@@ -263,14 +271,26 @@ struct StarTB {
                                            float2 (&done)[VY][2], const unsigned (&mz)[R + 1]) {
         // x neighbours beyond my 4 cells, from the adjacent lanes
         float lft[VY][4], rgt[VY][4];
+        if constexpr (L == 0 && R >= 3) {
+            // (two vector loads of the staged row in place of 2R shuffles:
+            // radius 4, one level, 768^3 460 -> 480 Gcell-steps/s)
 #pragma unroll
-        for (int y = 0; y < VY; ++y)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const float me = (e & 1) ? v[y][e >> 1].y : v[y][e >> 1].x;
-                lft[y][e] = (e >= 4 - R) ? __shfl_up_sync(0xffffffffu, me, 1) : 0.f;
-                rgt[y][e] = (e < R) ? __shfl_down_sync(0xffffffffu, me, 1) : 0.f;
+            for (int y = 0; y < VY; ++y) {
+                const float4 l4 = lds4(rows + (my_row + y + R) * pitch + col - 4);
+                const float4 r4 = lds4(rows + (my_row + y + R) * pitch + col + 4);
+                lft[y][0] = l4.x; lft[y][1] = l4.y; lft[y][2] = l4.z; lft[y][3] = l4.w;
+                rgt[y][0] = r4.x; rgt[y][1] = r4.y; rgt[y][2] = r4.z; rgt[y][3] = r4.w;
             }
+        } else {
+#pragma unroll
+            for (int y = 0; y < VY; ++y)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float me = (e & 1) ? v[y][e >> 1].y : v[y][e >> 1].x;
+                    lft[y][e] = (e >= 4 - R) ? __shfl_up_sync(0xffffffffu, me, 1) : 0.f;
+                    rgt[y][e] = (e < R) ? __shfl_down_sync(0xffffffffu, me, 1) : 0.f;
+                }
+        }
         // y neighbours outside my VY rows, from shared memory
         float4 up[VY][R], dn[VY][R];
 #pragma unroll
@@ -294,44 +314,47 @@ struct StarTB {
             const float4 q = (j < 0) ? up[y][-j - 1] : dn[y][j - 1];
             return h ? make_float2(q.z, q.w) : make_float2(q.x, q.y);
         };
-        // target t is plane zp - R + t, kept in slot (PHL - R + t) mod 2R;
-        // cells go in x pairs through packed FP32x2 FMAs (each lane an
-        // ordinary fused multiply-add, so the per-cell order is unchanged)
+        // target t (t = 0..2R) is plane zp - R + t.  Unrolled 2R times its slot
+        // is fixed, (PHL - R + t) mod 2R, and target 2R starts in the slot
+        // target 0 leaves; otherwise it is slot t, and every sum moves one
+        // slot down as this arrival's last product is added (a name: the
+        // FMA's destination).  Cells go in x pairs through packed FP32x2 FMAs
+        // (each lane an ordinary fused multiply-add, so the per-cell order is
+        // unchanged)
+        constexpr bool FIX = S::UNR == W2;
+        auto src = [](int t) constexpr { return FIX ? pmod(PHL - R + t, W2) : t; };
+        auto dst = [](int t) constexpr { return FIX ? pmod(PHL - R + t, W2) : t - 1; };
 #pragma unroll
         for (int y = 0; y < VY; ++y)
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int e0 = 2 * h;
                 const float2 x = v[y][h];
-#pragma unroll
-                for (int t = R + 1; t < 2 * R; ++t) {
-                    float2& acc = A[L][pmod(PHL - R + t, W2)][y][h];
-                    acc = __ffma2_rn(a.cf2[cidx<R>(0, -1, t - R)], x, acc);
-                }
-                {
-                    float2& acc = A[L][pmod(PHL, W2)][y][h];
-                    float2 s2 = __ffma2_rn(a.cf2[0], x, acc);
-#pragma unroll
-                    for (int j = 1; j <= R; ++j) {
-                        s2 = __ffma2_rn(a.cf2[cidx<R>(1, -1, j)], ypair(y, -j, h), s2);
-                        s2 = __ffma2_rn(a.cf2[cidx<R>(1, +1, j)], ypair(y, +j, h), s2);
-                    }
-#pragma unroll
-                    for (int j = 1; j <= R; ++j) {
-                        s2 = __ffma2_rn(a.cf2[cidx<R>(2, -1, j)], xpair(y, e0 - j), s2);
-                        s2 = __ffma2_rn(a.cf2[cidx<R>(2, +1, j)], xpair(y, e0 + j), s2);
-                    }
-                    // a boundary target keeps the value of its centre arrival
-                    acc = pick<MODE>(mz[R], y, h, x, s2);
-                }
+                const float2 a0 = A[L][src(0)][y][h];
+                done[y][h] = pick<MODE>(mz[0], y, h, a0, __ffma2_rn(a.cf2[cidx<R>(0, +1, R)], x, a0));
 #pragma unroll
                 for (int t = 1; t < R; ++t) {
-                    float2& acc = A[L][pmod(PHL - R + t, W2)][y][h];
-                    acc = pick<MODE>(mz[t], y, h, acc, __ffma2_rn(a.cf2[cidx<R>(0, +1, R - t)], x, acc));
+                    const float2 acc = A[L][src(t)][y][h];
+                    A[L][dst(t)][y][h] = pick<MODE>(mz[t], y, h, acc, __ffma2_rn(a.cf2[cidx<R>(0, +1, R - t)], x, acc));
                 }
-                float2& a0 = A[L][pmod(PHL - R, W2)][y][h];
-                done[y][h] = pick<MODE>(mz[0], y, h, a0, __ffma2_rn(a.cf2[cidx<R>(0, +1, R)], x, a0));
-                a0 = __fmul2_rn(a.cf2[cidx<R>(0, -1, R)], x);  // first contribution to target zp + R
+                float2 s2 = __ffma2_rn(a.cf2[0], x, A[L][src(R)][y][h]);
+#pragma unroll
+                for (int j = 1; j <= R; ++j) {
+                    s2 = __ffma2_rn(a.cf2[cidx<R>(1, -1, j)], ypair(y, -j, h), s2);
+                    s2 = __ffma2_rn(a.cf2[cidx<R>(1, +1, j)], ypair(y, +j, h), s2);
+                }
+#pragma unroll
+                for (int j = 1; j <= R; ++j) {
+                    s2 = __ffma2_rn(a.cf2[cidx<R>(2, -1, j)], xpair(y, e0 - j), s2);
+                    s2 = __ffma2_rn(a.cf2[cidx<R>(2, +1, j)], xpair(y, e0 + j), s2);
+                }
+                // a boundary target keeps the value of its centre arrival
+                A[L][dst(R)][y][h] = pick<MODE>(mz[R], y, h, x, s2);
+#pragma unroll
+                for (int t = R + 1; t < 2 * R; ++t)
+                    A[L][dst(t)][y][h] = __ffma2_rn(a.cf2[cidx<R>(0, -1, t - R)], x, A[L][src(t)][y][h]);
+                // first contribution to target zp + R
+                A[L][FIX ? src(0) : 2 * R - 1][y][h] = __fmul2_rn(a.cf2[cidx<R>(0, -1, R)], x);
             }
     }
 
@@ -366,8 +389,7 @@ struct StarTB {
         }
     }
 
-    // level L of phase p (PH = p mod 2R; p0 is a multiple of 2R, so the
-    // parity of p is that of PH): consumes input plane za + p (L = 0) or what
+    // level L of phase p (PH = p mod UNR): consumes input plane za + p (L = 0) or what
     // level L-1 completed in phase p-1 (plane za + p - L(R+1))
     template <int L, int PH, int MODE>
     __device__ __forceinline__ void level_body(int p) {
@@ -376,7 +398,7 @@ struct StarTB {
 #pragma unroll
         for (int t = 0; t <= R; ++t) mz[t] = MODE == kBndCells ? bmask(zp - R + t) : 0u;
         float2 v[VY][2], done[VY][2];
-        constexpr int PHL = pmod(PH - L * (R + 1), W2);
+        constexpr int PHL = pmod(PH - L * (R + 1), S::UNR);
         if constexpr (L == 0) {
             const T* rows = sin + ((gb + p) % NI) * (SLOT / ES);
 #pragma unroll
@@ -387,7 +409,7 @@ struct StarTB {
             }
             arrive<0, PHL, MODE>(v, rows, LXB, col0, done, mz);
         } else {
-            const float* prev = slev + ((L - 1) * NB + ((PH + 1) & 1)) * ROWS * LX;  // slot of phase p-1
+            const float* prev = slev + ((L - 1) * NB + ((p + 1) & 1)) * ROWS * LX;  // slot of phase p-1
 #pragma unroll
             for (int y = 0; y < VY; ++y) {
                 if constexpr (S::CARRY) {
@@ -406,7 +428,7 @@ struct StarTB {
         } else {
             // my cells stay in registers for level L+1; the shared-memory plane
             // serves the neighbouring warps (the R rows at each end)
-            float* lb = slev + (L * NB + (PH & 1)) * ROWS * LX;
+            float* lb = slev + (L * NB + (p & 1)) * ROWS * LX;
 #pragma unroll
             for (int y = 0; y < VY; ++y) {
                 if (!S::CARRY || y < R || y >= VY - R)
@@ -436,7 +458,7 @@ struct StarTB {
     }
 
     // phase p = p0 + PH; false when an input copy did not land in time
-    // the levels of phase p (PH = p mod 2R)
+    // the levels of phase p (PH = p mod UNR)
     template <int PH>
     __device__ __forceinline__ void phase_levels(int p) {
         // the arrivals of this phase span planes za + p - (K-1)(R+1) .. za + p;
@@ -451,8 +473,7 @@ struct StarTB {
             else if (fixed || wmode != kBndNone) levels<K - 1, PH, kBndCells, false>(p, all);
             else levels<K - 1, PH, kBndNone, false>(p, all);
         } else {
-            // long bodies (2R phases of them): one body per boundary mode,
-            // which keeps the loop inside the instruction cache
+            // long bodies: one per boundary mode
             if (fixed || wmode == kBndCells) levels<K - 1, PH, kBndCells, false>(p, all);
             else if (wmode == kBndColumns) levels<K - 1, PH, kBndColumns, false>(p, all);
             else levels<K - 1, PH, kBndNone, false>(p, all);
@@ -471,7 +492,7 @@ struct StarTB {
             stage_ragged(p + PD);
             cp_async_commit();
             phase_levels<PH>(p);
-            if constexpr (PH + 1 < W2) return phase<PH + 1>(p0);
+            if constexpr (PH + 1 < S::UNR) return phase<PH + 1>(p0);
             return true;
         }
         const int g = (gb + p) % NI;
@@ -500,7 +521,7 @@ struct StarTB {
             issue(p + PD);
         }
         phase_levels<PH>(p);
-        if constexpr (PH + 1 < W2) return phase<PH + 1>(p0);
+        if constexpr (PH + 1 < S::UNR) return phase<PH + 1>(p0);
         return true;
     }
 
@@ -570,7 +591,7 @@ struct StarTB {
         }
         // last arrival any level needs: level K-1 at plane need_hi + R - 1
         const int nph0 = (need_hi + R - 1 - za) + (K - 1) * (R + 1) + 1;
-        const int nph = (nph0 + W2 - 1) / W2 * W2;
+        const int nph = (nph0 + S::UNR - 1) / S::UNR * S::UNR;
         // (the slots were last read through the generic proxy by the previous
         // piece, behind the barrier that ended it)
         if (threadIdx.x == 0) fence_proxy_async_smem();
@@ -587,7 +608,7 @@ struct StarTB {
             }
         }
         bool ok = true;
-        for (int p0 = 0; p0 < nph && ok; p0 += W2) ok = phase<0>(p0);
+        for (int p0 = 0; p0 < nph && ok; p0 += S::UNR) ok = phase<0>(p0);
         return ok;
     }
 
