@@ -132,6 +132,9 @@ int shape_of(const Plan& p) {
     return p.ndim == 3 ? kStar3D : kStar2D;
 }
 
+// Largest pitch of a 2D copy (cudaDevAttrMaxPitch of every device so far).
+constexpr int64_t kMaxPitch = 0x7fffffff;
+
 // Copies planes [lo, hi) between host and a (possibly circular) device buffer.
 cudaError_t copy_planes(const Buffer& b, char* arena, char* host, int64_t host_plane_bytes,
                         int64_t host_field_bytes, int nfields, int64_t lo, int64_t hi, int64_t slot0,
@@ -141,16 +144,25 @@ cudaError_t copy_planes(const Buffer& b, char* arena, char* host, int64_t host_p
     int64_t fstride = b.cap * pb;            // device bytes between fields
     int64_t s0 = slot0 % b.cap;
     int64_t first = std::min(n, b.cap - s0);
-    for (int f = 0; f < nfields; ++f) {
-        char* h = host + f * host_field_bytes + lo * host_plane_bytes;
-        char* d = arena + b.offset + f * fstride;
-        int64_t segs[2][3] = {{s0, 0, first}, {0, first, n - first}};
-        for (auto& sg : segs) {
-            if (sg[2] <= 0) continue;
-            char* dp = d + sg[0] * pb;
-            char* hp = h + sg[1] * host_plane_bytes;
-            cudaError_t e = to_device ? cudaMemcpyAsync(dp, hp, sg[2] * pb, cudaMemcpyHostToDevice, s)
-                                      : cudaMemcpyAsync(hp, dp, sg[2] * pb, cudaMemcpyDeviceToHost, s);
+    const int64_t segs[2][3] = {{s0, 0, first}, {0, first, n - first}};
+    for (auto& sg : segs) {
+        if (sg[2] <= 0) continue;
+        char* dp = arena + b.offset + sg[0] * pb;
+        char* hp = host + (lo + sg[1]) * host_plane_bytes;
+        // the fields of a segment lie at constant strides on both sides: one
+        // 2D copy of nfields rows (a row is contiguous planes) in place of
+        // nfields calls; strides beyond the copy engines' pitch go one by one
+        if (nfields > 1 && fstride <= kMaxPitch && host_field_bytes <= kMaxPitch) {
+            cudaError_t e = to_device
+                ? cudaMemcpy2DAsync(dp, fstride, hp, host_field_bytes, sg[2] * pb, nfields, cudaMemcpyHostToDevice, s)
+                : cudaMemcpy2DAsync(hp, host_field_bytes, dp, fstride, sg[2] * pb, nfields, cudaMemcpyDeviceToHost, s);
+            if (e != cudaSuccess) return e;
+            continue;
+        }
+        for (int f = 0; f < nfields; ++f) {
+            char *d = dp + f * fstride, *h = hp + f * host_field_bytes;
+            cudaError_t e = to_device ? cudaMemcpyAsync(d, h, sg[2] * pb, cudaMemcpyHostToDevice, s)
+                                      : cudaMemcpyAsync(h, d, sg[2] * pb, cudaMemcpyDeviceToHost, s);
             if (e != cudaSuccess) return e;
         }
     }
