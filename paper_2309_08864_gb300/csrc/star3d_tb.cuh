@@ -345,8 +345,18 @@ struct StarTB {
                 }
 #pragma unroll
                 for (int j = 1; j <= R; ++j) {
-                    s2 = __ffma2_rn(a.cf2[cidx<R>(2, -1, j)], xpair(y, e0 - j), s2);
-                    s2 = __ffma2_rn(a.cf2[cidx<R>(2, +1, j)], xpair(y, e0 + j), s2);
+                    if (j % 2 == 0) {
+                        s2 = __ffma2_rn(a.cf2[cidx<R>(2, -1, j)], xpair(y, e0 - j), s2);
+                        s2 = __ffma2_rn(a.cf2[cidx<R>(2, +1, j)], xpair(y, e0 + j), s2);
+                    } else {
+                        // pairs that start at an odd column would have to be
+                        // put together first: two scalar FMAs instead
+                        const float cm = a.cf[cidx<R>(2, -1, j)], cp = a.cf[cidx<R>(2, +1, j)];
+                        s2.x = __fmaf_rn(cm, xval(y, e0 - j), s2.x);
+                        s2.y = __fmaf_rn(cm, xval(y, e0 + 1 - j), s2.y);
+                        s2.x = __fmaf_rn(cp, xval(y, e0 + j), s2.x);
+                        s2.y = __fmaf_rn(cp, xval(y, e0 + 1 + j), s2.y);
+                    }
                 }
                 // a boundary target keeps the value of its centre arrival
                 A[L][dst(R)][y][h] = pick<MODE>(mz[R], y, h, x, s2);
