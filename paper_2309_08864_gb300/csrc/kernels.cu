@@ -4,6 +4,7 @@
 #include "plane_tb.cuh"
 #include "row2d_tb.cuh"
 #include "star3d_tb.cuh"
+#include "tile2d_tb.cuh"
 
 #include <cmath>
 #include <cstdlib>
@@ -317,6 +318,44 @@ void choose_row_split(LaunchShape& ls, int64_t nout, int r, int depth, int csize
     ls.grid.x = (unsigned)((strips * (a.split + a.split2) + kRowWarps - 1) / kRowWarps);
 }
 
+bool tile2d_short(LaunchShape& ls, int shape, int64_t nout, int64_t nx, int r, int depth, int csize, int sms) {
+    // Rows of 32 columns per SM up to which the tile is the faster one
+    // (in-core Gcell-steps/s, strips / tile).  FP64, fused: 80x512 radius 1, 4
+    // levels 5.6 / 15.7, 512^2 28 / 43, 1024^2 60 / 73 (215 rows per SM); one
+    // level has little halo to save (512^2 20.9 / 20.3).  FP32: 81-point box,
+    // one level 512^2 14.0 / 18.8, 1024^2 49 / 52; radius 3, 4 levels,
+    // 701x1003 93 / 106; 9-point box, 8 levels 512^2 74 / 85 (54 rows), 1024^2
+    // 272 / 219; radius 1, 4 levels 80x512 18 / 20, 256^2 (13 rows) 26 / 25,
+    // 512^2 94 / 72.
+    const int H = r * depth;
+    const int64_t limit = csize == 8 ? (depth > 1 ? 256 : 0)
+                          : (shape == kBox2D && r >= 3) || H >= 12 ? 160
+                          : H >= 6 ? 60 : depth > 1 ? 12 : 0;
+    const int64_t gx = (nx + kTileX - 1) / kTileX;
+    if (sms <= 0 || nout <= 0 || gx * nout > limit * sms) return false;
+    double best = 0;
+    int best_ty = 0;
+    for (int ty = 4; ty <= 64; ++ty) {
+        if (tile2d_smem(r, depth, ty, csize) > kSmemLimit) break;
+        const int64_t gy = (nout + ty - 1) / ty;
+        if (gy > 65535) continue;
+        double work = 0;
+        for (int l = 1; l <= depth; ++l) work += (double)(kTileX + 2 * (H - l * r)) * (ty + 2 * (H - l * r));
+        const double cost = (double)((gx * gy + sms - 1) / sms) * (work + 256.0);
+        if (!best_ty || cost < best) { best_ty = ty; best = cost; }
+    }
+    if (!best_ty) return false;
+    ls.lx = kTileX + 2 * H;
+    ls.ly = best_ty + 2 * H;
+    ls.tx = kTileX;
+    ls.ty = best_ty;
+    ls.block = dim3(kTileThreads, 1, 1);
+    ls.smem = (size_t)tile2d_smem(r, depth, best_ty, csize);
+    ls.grid = dim3((unsigned)gx, (unsigned)((nout + best_ty - 1) / best_ty), 1);
+    ls.fast = kFastTile2D;
+    return true;
+}
+
 cudaError_t launch_stencil(int dtype, int shape, int r, const StencilArgs& a, const LaunchShape& ls,
                            cudaStream_t s) {
     if (ls.fast == kFastStar3D) switch (dtype) {
@@ -325,7 +364,7 @@ cudaError_t launch_stencil(int dtype, int shape, int r, const StencilArgs& a, co
         case SO2DR_F16: return ls.ragged ? launch_star3d_ragged_f16(r, a, ls, s) : launch_star3d_f16(r, a, ls, s);
         default: return cudaErrorInvalidValue;
     }
-    if (ls.fast == kFastRow2D) switch (dtype) {
+    if (ls.fast == kFastRow2D || ls.fast == kFastTile2D) switch (dtype) {
         case SO2DR_F64: return launch_row2d_f64(shape, r, a, ls, s);
         case SO2DR_F32: return launch_row2d_f32(shape, r, a, ls, s);
         case SO2DR_BF16: return launch_row2d_bf16(shape, r, a, ls, s);

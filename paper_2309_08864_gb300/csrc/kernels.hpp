@@ -16,11 +16,11 @@ struct LaunchShape {
     int lx, ly, tx, ty;
     bool ok;
     int fast;    // 0 generic kernel, kFastStar3D (star3d_tb.cuh), kFastRow2D (row2d_tb.cuh),
-                 // kFastBox2D (box2d_fast.cuh), kFastPlane3D (plane_tb.cuh)
+                 // kFastBox2D (box2d_fast.cuh), kFastPlane3D (plane_tb.cuh), kFastTile2D (tile2d_tb.cuh)
     bool ragged; // rows are not whole 4-element vectors: the kernels' element-wise staging
 };
 
-constexpr int kFastStar3D = 1, kFastRow2D = 2, kFastBox2D = 3, kFastPlane3D = 4;
+constexpr int kFastStar3D = 1, kFastRow2D = 2, kFastBox2D = 3, kFastPlane3D = 4, kFastTile2D = 5;
 
 // Axes the register-streaming kernels index with 32-bit integers end here;
 // longer ones run on the generic kernel.
@@ -86,6 +86,10 @@ void choose_work_split(LaunchShape& ls, int64_t nout, int r, int depth, int sms,
 // (axis-0 segments per strip) and ls.grid.x (the strips before the call, the
 // CTAs after it).
 void choose_row_split(LaunchShape& ls, int64_t nout, int r, int depth, int csize, int sms, int occ, StencilArgs& a);
+
+// Replaces a 2D launch of few rows by the shared-memory tile kernel where that
+// is rated faster; false: keep ls.
+bool tile2d_short(LaunchShape& ls, int shape, int64_t nout, int64_t nx, int r, int depth, int csize, int sms);
 
 // 3D star kernel (star3d_tb.cuh), a translation unit per storage type and
 // kind of rows.

@@ -159,7 +159,10 @@ extern "C" int so2dr_run_device_noalloc(int ndim, const int64_t* dims, int radiu
         ls.grid.z = 1;
         StencilArgs a;
         std::memset(&a, 0, sizeof(a));
-        if (ls.fast && ls.fast != kFastPlane3D) {
+        if (ls.fast == kFastRow2D) tile2d_short(ls, shape, n0, nx, radius, depth, csize, sms);
+        if (ls.fast == kFastTile2D) {
+            // (its grid is its tiles)
+        } else if (ls.fast && ls.fast != kFastPlane3D) {
             int occ = stencil_occupancy(dtype, shape, radius, depth, ls);
             if (ls.fast == kFastStar3D) choose_work_split(ls, n0, radius, depth, sms, occ, &a.split);
             else if (ls.fast == kFastBox2D) ls.grid.z = (unsigned)choose_segments((int64_t)ls.grid.x * ls.grid.y, n0, radius, depth, sms, occ, false);

@@ -189,6 +189,7 @@ int enqueue_stencil(so2dr_plan_s* P, const RunList& rl, const Op& op, cudaStream
     const Buffer& bo = rl.bufs[o.dst_buf];
     if (o.src_hi - o.src_lo > bi.cap || o.dst_slot0 < 0 || o.dst_slot0 + (o.dst_hi - o.dst_lo) > bo.cap)
         return set_error(SO2DR_E_DEVICE_CHECK, "kernel op exceeds its buffer");
+    if (ls.fast == kFastRow2D) tile2d_short(ls, shape, o.dst_hi - o.dst_lo, p.nx, p.r, o.depth, csize, P->sm_count);
     StencilArgs a;
     std::memset(&a, 0, sizeof(a));
     a.in = P->arena + bi.offset;
@@ -231,7 +232,9 @@ int enqueue_stencil(so2dr_plan_s* P, const RunList& rl, const Op& op, cudaStream
         a.cf[k] = (float)p.coeffs[k];
         a.cf2[k] = make_float2(a.cf[k], a.cf[k]);
     }
-    if (ls.fast && ls.fast != kFastPlane3D) {
+    if (ls.fast == kFastTile2D) {
+        // (its grid is its tiles)
+    } else if (ls.fast && ls.fast != kFastPlane3D) {
         // split the work so that the grid fills the SMs evenly
         int& occ = P->occ_cache[1][o.depth];
         if (!occ) occ = stencil_occupancy(p.dtype, shape, p.r, o.depth, ls);
