@@ -157,12 +157,15 @@ LaunchShape stencil_launch_shape(int shape, int r, int depth, int64_t n0, int64_
         }
         if (ls.ok) return ls;
     }
-    if (fast_ok && ny * nx <= kMaxFastAxis && (shape == kVarcoef3D || (shape == kStar3D && csize == 8))) {
+    int H = r * depth;
+    // (only depths the generic kernel takes too, so that the deepest supported
+    // launch does not depend on the kernel)
+    if (fast_ok && ny * nx <= kMaxFastAxis && (shape == kVarcoef3D || (shape == kStar3D && csize == 8)) &&
+        stencil_smem_bytes(shape, r, depth, tile_edge(H), tile_edge(H), csize) <= kSmemLimit) {
         plane_shape(ls, r, depth, ny, nx, csize);
         if (ls.ok) return ls;
         ls.fast = 0;
     }
-    int H = r * depth;
     if (is3d(shape)) {
         ls.lx = ls.ly = tile_edge(H);
         ls.tx = ls.lx - 2 * H;
