@@ -4,11 +4,13 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
+#include <initializer_list>
 #include <limits>
 
 namespace so2dr {
 
 bool fast_star3d_supported(int r, int depth);
+int choose_segments(int64_t tiles, int64_t nout, int r, int depth, int sms, int occ, bool share_sm);
 bool fast_star3d_row_ok(int64_t nx, int esize);
 
 
@@ -594,6 +596,66 @@ double kernel_rate(const Plan& p, int depth) {
     return depth >= 2 ? 112e9 : 429e9;
 }
 
+// Rates of the FP32 and FP64 constant-coefficient kernels (in-core cell updates
+// per second on one GB300, 1024^3 and 768^3 FP32 stars, 12800^2 boxes, 8192^2
+// stars; depths in between interpolated).  FP64 is bound by the FP64 units
+// (0.38 T FMA/s reached), less the recomputed halo of fused levels.
+double kernel_rate_now(const Plan& p, int depth) {
+    auto at = [&](std::initializer_list<double> v) { return *(v.begin() + std::min<int>(depth, (int)v.size()) - 1) * 1e9; };
+    if (p.dtype == SO2DR_F64) {
+        const double pts = num_coeffs(p.ndim, p.r, p.kind);
+        if (p.ndim == 2 && depth > (p.r <= 2 ? 4 : 2)) return 10e9;  // the generic kernel
+        return 0.38e12 / pts * (p.ndim == 2 ? 1.0 - 2.0 * p.r * depth / 128.0 : depth > 4 ? 0.5 : depth > 1 ? 0.72 : 1.0);
+    }
+    if (p.ndim == 3) {
+        if (!fast_star3d_supported(p.r, depth)) return 60e9;
+        switch (p.r) {
+            case 1: return at({815, 1323, 1494, 1565});
+            case 2: return at({703, 885});
+            case 3: return at({528, 376});
+            default: return at({494, 258});
+        }
+    }
+    const double ragged = p.nx % 4 ? 0.8 : 1.0;
+    if (p.kind == SO2DR_BOX) switch (p.r) {
+        // (fused depths as they compare out of core, 12800^2, 640 steps: 8 levels
+        // 76.8 ms, 6 79.0, 5 79.2, 4 82.1)
+        case 1: return depth > 8 ? 50e9 : ragged * at({763, 1200, 1450, 1649, 1690, 1714, 1740, 1763});
+        case 2: return depth > 4 ? 50e9 : ragged * at({730, 759, 799, 825});
+        case 3: return depth > 3 ? 50e9 : ragged * at({481, 408, 403});
+        default: return depth > 2 ? 40e9 : ragged * at({321, 287});
+    }
+    if (depth > (p.r == 1 ? 8 : 4)) return 40e9;
+    switch (p.r) {
+        case 1: return ragged * at({700, 1250, 1700, 2050, 2030, 2000, 1950, 1900});
+        case 2: return ragged * at({650, 950, 1050, 1050});
+        case 3: return ragged * at({600, 700, 720, 700});
+        default: return ragged * at({550, 600, 580, 545});
+    }
+}
+
+// Time of one launch that writes `planes` planes.  A segment streams the halo
+// and the pipeline's fill beside its own planes; the 3D star kernel's CTAs
+// (tiles x segments) are counted per SM, as its work split does.
+double launch_seconds(const Plan& p, int depth, double planes) {
+    const double fixed = 5e-6;  // launch, staging latency, tail
+    const double rate = kernel_rate_now(p, depth);
+    if (p.ndim == 3 && p.dtype == SO2DR_F32 && fast_star3d_supported(p.r, depth)) {
+        const int sms = 152;
+        const int64_t tx = 128 - 2 * ((p.r * depth + 3) / 4 * 4);
+        const int64_t ty = (depth == 1 || p.r >= 3 ? 16 : 32) - 2 * p.r * (depth - 1);
+        const int64_t edge = p.r <= 2 ? 1024 : 768;  // the grid the rate was measured on
+        const double ovh = 2.0 * p.r * depth + depth;
+        const double tiles0 = (double)((edge + tx - 1) / tx) * (double)((edge + ty - 1) / ty);
+        const double tau = (double)edge * edge * depth / rate * sms / tiles0;  // an SM's time per plane of a tile
+        const int64_t tiles = ((p.nx + tx - 1) / tx) * ((p.ny + ty - 1) / ty);
+        const int n = choose_segments(tiles, (int64_t)std::max(1.0, planes), p.r, depth, sms, 1, true);
+        return fixed + (double)((tiles * n + sms - 1) / sms) * (planes / n + ovh) * tau;
+    }
+    const double halo = p.ndim == 3 ? (double)depth * (p.r + 1) : (double)p.r * depth;
+    return fixed + (planes + halo) * (double)p.plane_cells * depth / rate;
+}
+
 double predict_ms(const Plan& p) {
     double comp, use;
     trapezoid_work(p, &comp, &use);
@@ -608,8 +670,22 @@ double predict_ms(const Plan& p) {
     // single-step launches keep the in-core rate
     const double pavg = (double)p.interior_planes() / std::max(1, p.d);
     const double eff = p.k_on > 1 ? std::max(0.6, pavg / (pavg + 15.0)) : 1.0;
-    const double kernel = comp * cells_plane / (eff * kernel_rate(p, p.k_on));
-    const int L = (int)launch_depths(p.k_off, p.k_on).size();
+    double kernel = comp * cells_plane / (eff * kernel_rate(p, p.k_on));
+    const std::vector<int> depths = launch_depths(p.k_off, p.k_on);
+    const int L = (int)depths.size();
+    // Where the planner chooses the round length: launch by launch, for a chunk
+    // away from the grid's ends.  (FP32 and FP64 only, whose results do not
+    // depend on the depths: 16-bit storage rounds at every launch's end, and
+    // its plans, with them its results, stay what they were.)
+    if (p.auto_rounds && !vc && (p.dtype == SO2DR_F32 || p.dtype == SO2DR_F64)) {
+        double chunk = 0;
+        int m = 0;
+        for (int dl : depths) {
+            m += dl;
+            chunk += launch_seconds(p, dl, std::min((double)p.n0, pavg + 2.0 * p.r * (p.k_off - m)));
+        }
+        kernel = chunk * (double)p.d * (double)p.T / (double)p.k_off;
+    }
     const double units = (double)std::max(1, p.d * p.rounds);
     const double t_launch = kernel / (units * L), t_d2h_chunk = host_d2h / units;
     // without look-ahead a chunk's transfer waits for the previous chunk's
@@ -706,6 +782,7 @@ int build_plan(Plan& p, int ndim, const int64_t* dims, int radius, int kind, con
     if (bw_h2d > 0) p.bw_h2d = bw_h2d;
     if (bw_d2h > 0) p.bw_d2h = bw_d2h;
     if (bw_hbm > 0) p.bw_hbm = bw_hbm;
+    p.auto_rounds = k_off == 0;
     if (p.n0 - 2 * p.r < 1) {
         // no interior plane: nothing ever changes; a one-chunk plan with no rounds
         p.k_off = std::max(1, k_off);
