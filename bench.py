@@ -46,7 +46,7 @@ sys.path.insert(0, ROOT)
 
 MEASURED = os.path.join(ROOT, "MEASURED_PEAKS.json")
 KERNEL_SRC = {"star": os.path.join(ROOT, "paper_2309_08864_gb300", "csrc", "star3d_tb.cuh"),
-              "box": os.path.join(ROOT, "paper_2309_08864_gb300", "csrc", "box2d_fast.cuh")}
+              "box": os.path.join(ROOT, "paper_2309_08864_gb300", "csrc", "row2d_tb.cuh")}
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per k_on-deep launch
 # of the benchmarked plan, from one ncu capture of the benchmark command (the
 # summaries under profiles/ give the commands), keyed by the first 16 hex
@@ -690,7 +690,8 @@ def bench_config(args, cfg, name, world, rank, local, torch, inputs, so2dr, link
                      "traffic_vs_alg": traffic / alg_bytes_per_launch if traffic and alg_bytes_per_launch else None,
                      "traffic_read_vs_alg": cap[4] / (alg_bytes_per_launch / 2) if traffic and alg_bytes_per_launch else None,
                      "traffic_write_vs_alg": cap[5] / (alg_bytes_per_launch / 2) if traffic and alg_bytes_per_launch else None,
-                     "kernel": ("box2d_fast_kernel" if kind == "box" else "star3d_tb_kernel")
+                     "kernel": ("star3d_tb_kernel" if kind != "box" else
+                                "box2d_fast_kernel" if (cfg["r"], info["k_on"]) == (2, 4) else "row2d_tb_kernel")
                                + " (k_on-step TB launch)", "peak_kind": ("derived from unit counts and the maximum SM clock" if alu_bound
                                    else peak_kind + " (burst)"),
                      "alg_bytes_per_launch": alg_bytes_per_launch,

@@ -3,7 +3,8 @@
 // arithmetic on FP32 / BF16 / FP16 storage.
 //
 // The on-chip temporal blocking of Sec. III / Sec. IV-A for the paper's
-// box2d workloads (Table III), laid out for sm_103a:
+// box2d workloads (Table III), laid out for sm_103a.  Launched at radius 2, four
+// levels (wide_box2d in kernels.cu); the other depths run row2d_tb.cuh.
 //  * a CTA owns a strip of 1024 columns (256 threads x 4 columns) and streams
 //    the rows of axis 0 through it; axis 0 may be split into segments
 //    (gridDim.z) so that the grid fills the SMs;
@@ -60,10 +61,6 @@ struct FastBox {
                          NBI = S::NBI;
     static constexpr int W2 = 2 * R, WD = 2 * R + 1;
     static constexpr int NF = 12;  // window: columns -4..7 around my first column
-    // accumulation loop order (same results): column offset outer for small
-    // R*K, target outer for larger ones (measured on 16384^2: offset-outer
-    // 14-28% faster up to R*K = 4, 2-15% slower from 8)
-    static constexpr bool kOffsetOuter = R * K <= 4;
 
     const StencilArgs& a;
     T* sin;       // [NBI][ROW] staged input rows (row of phase p in slot p % NBI)
@@ -99,52 +96,23 @@ struct FastBox {
         for (int j = 4 - R; j <= 6 + R; ++j) P[j] = make_float2(f[j], f[j + 1]);
         // target q (q = 0..2R) is row y' - R + q, its slot (PH - R + q) mod 2R;
         // this arrival is its coefficient row 2R - q; target 2R (row y' + R)
-        // starts in the slot target 0 leaves.  Every target adds its products
-        // in ascending column order whichever loop is outer.
-        if constexpr (kOffsetOuter) {
-            // column offset outer: the 2(2R+1) accumulators of one step are
-            // independent (faster while R*K <= 4 leaves the registers for it)
-            float2 acc[W2 + 1][2];
+        // starts in the slot target 0 leaves.  One accumulator chain at a time.
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
+        for (int h = 0; h < 2; ++h) {
 #pragma unroll
-                for (int q = 0; q < W2; ++q) acc[q][h] = A[L][pmod(PH - R + q, W2)][h];
-                acc[W2][h] = __fmul2_rn(a.cf2[0], P[2 * h - R + 4]);
+            for (int q = 0; q < W2; ++q) {
+                float2& acc = A[L][pmod(PH - R + q, W2)][h];
+                float2 s2 = acc;
+#pragma unroll
+                for (int dx = -R; dx <= R; ++dx)
+                    s2 = __ffma2_rn(a.cf2[(W2 - q) * WD + dx + R], P[2 * h + dx + 4], s2);
+                if (q == 0) done[h] = s2;
+                else acc = s2;
             }
+            float2 s2 = __fmul2_rn(a.cf2[0], P[2 * h - R + 4]);
 #pragma unroll
-            for (int dx = -R; dx <= R; ++dx)
-#pragma unroll
-                for (int q = 0; q <= W2; ++q)
-#pragma unroll
-                    for (int h = 0; h < 2; ++h)
-                        if (q < W2 || dx > -R)
-                            acc[q][h] = __ffma2_rn(a.cf2[(W2 - q) * WD + dx + R], P[2 * h + dx + 4], acc[q][h]);
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                done[h] = acc[0][h];
-#pragma unroll
-                for (int q = 1; q < W2; ++q) A[L][pmod(PH - R + q, W2)][h] = acc[q][h];
-                A[L][pmod(PH - R, W2)][h] = acc[W2][h];
-            }
-        } else {
-            // target outer: one accumulator chain at a time (fewer live registers)
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-#pragma unroll
-                for (int q = 0; q < W2; ++q) {
-                    float2& acc = A[L][pmod(PH - R + q, W2)][h];
-                    float2 s2 = acc;
-#pragma unroll
-                    for (int dx = -R; dx <= R; ++dx)
-                        s2 = __ffma2_rn(a.cf2[(W2 - q) * WD + dx + R], P[2 * h + dx + 4], s2);
-                    if (q == 0) done[h] = s2;
-                    else acc = s2;
-                }
-                float2 s2 = __fmul2_rn(a.cf2[0], P[2 * h - R + 4]);
-#pragma unroll
-                for (int dx = -R + 1; dx <= R; ++dx) s2 = __ffma2_rn(a.cf2[dx + R], P[2 * h + dx + 4], s2);
-                A[L][pmod(PH - R, W2)][h] = s2;
-            }
+            for (int dx = -R + 1; dx <= R; ++dx) s2 = __ffma2_rn(a.cf2[dx + R], P[2 * h + dx + 4], s2);
+            A[L][pmod(PH - R, W2)][h] = s2;
         }
     }
 
