@@ -98,8 +98,9 @@ void plane_shape(LaunchShape& ls, int r, int depth, int64_t ny, int64_t nx, int 
     ls.fast = kFastPlane3D;
 }
 
-template <int R, int K> void fast_shape(LaunchShape& ls, int64_t ny, int64_t nx, int esize) {
-    using S = StarShape<R, K>;
+template <int R, int K, bool SMALL = false> void fast_shape(LaunchShape& ls, int64_t ny, int64_t nx, int esize) {
+    using S = StarShape<R, K, SMALL>;
+    ls.small = SMALL;
     ls.lx = S::LX;
     ls.ly = S::LYT;
     ls.tx = S::TX;
@@ -118,7 +119,7 @@ LaunchShape stencil_launch_shape(int shape, int r, int depth, int64_t n0, int64_
     LaunchShape ls;
     ls.ok = false;
     ls.fast = 0;
-    ls.ragged = false;
+    ls.ragged = ls.small = false;
     if (depth < 1) return ls;
     const bool fast_ok = n0 <= kMaxFastAxis && ny <= kMaxFastAxis && nx <= kMaxFastAxis &&
                          !std::getenv("SO2DR_GENERIC_KERNEL");
@@ -281,6 +282,39 @@ void choose_work_split(LaunchShape& ls, int64_t nout, int r, int depth, int sms,
     } else {
         ls.grid.z = (unsigned)nseg;
     }
+}
+
+// Launches of up to this many cells take the 2-row tile (radius 1 fused, radius
+// 3 at one level).  In-core Gcell-steps/s, 4 rows / 2 rows: four levels 48x80x132
+// 89 / 96, 64^3 50 / 56, 101x99x97 117 / 151, 96^3 153 / 155, 128^3 252 / 186,
+// 160^3 two levels 329 / 298; radius 3 64^3 18.3 / 21.3, 128^3 111 / 99.
+constexpr double kSmallCells = 1e6;
+
+bool star_small(LaunchShape& ls, int64_t nout, int64_t ny, int64_t nx, int r, int depth, int esize, int sms) {
+    if (sms <= 0 || nout <= 0 || (double)nout * (double)ny * (double)nx > kSmallCells || std::getenv("SO2DR_WORK_SPLIT")) return false;
+    LaunchShape t = ls;
+    switch (r * 16 + depth) {
+        case 18: fast_shape<1, 2, true>(t, ny, nx, esize); break;
+        case 19: fast_shape<1, 3, true>(t, ny, nx, esize); break;
+        case 20: fast_shape<1, 4, true>(t, ny, nx, esize); break;
+        case 49: fast_shape<3, 1, true>(t, ny, nx, esize); break;
+        default: return false;
+    }
+    if (!t.ok) return false;
+    // A CTA's time goes with the planes it streams (segment, halo, pipeline
+    // fill); a second CTA on the same SM costs it about 60% more.
+    const double ovh = 2.0 * r * depth + depth;
+    const int64_t tiles = (int64_t)t.grid.x * t.grid.y;
+    double best = 0;
+    int best_n = 0;
+    for (int n = 1; n <= 64 && n <= nout; ++n) {
+        const int64_t c = (tiles * n + sms - 1) / sms;
+        const double cost = ((double)((nout + n - 1) / n) + ovh) * (3.6 * (double)(c / 2) + 2.2 * (double)(c % 2));
+        if (!best_n || cost < best * 0.98) { best_n = n; best = cost; }
+    }
+    t.grid.z = (unsigned)best_n;
+    ls = t;
+    return true;
 }
 
 void choose_row_split(LaunchShape& ls, int64_t nout, int r, int depth, int csize, int sms, int occ, StencilArgs& a) {

@@ -17,6 +17,7 @@ struct LaunchShape {
     bool ok;
     int fast;    // 0 generic kernel, kFastStar3D (star3d_tb.cuh), kFastRow2D (row2d_tb.cuh),
                  // kFastBox2D (box2d_fast.cuh), kFastPlane3D (plane_tb.cuh), kFastTile2D (tile2d_tb.cuh)
+    bool small;  // 3D star kernel: the 2-row tile (star_small)
     bool ragged; // rows are not whole 4-element vectors: the kernels' element-wise staging
 };
 
@@ -115,6 +116,10 @@ cudaError_t launch_row2d_f64(int shape, int r, const StencilArgs& a, const Launc
 cudaError_t launch_row2d_f32(int shape, int r, const StencilArgs& a, const LaunchShape& ls, cudaStream_t s);
 cudaError_t launch_row2d_bf16(int shape, int r, const StencilArgs& a, const LaunchShape& ls, cudaStream_t s);
 cudaError_t launch_row2d_f16(int shape, int r, const StencilArgs& a, const LaunchShape& ls, cudaStream_t s);
+
+// Gives a 3D star launch on a small grid the 2-row tile (sets ls, grid.z
+// included; grid split); false: keep ls.
+bool star_small(LaunchShape& ls, int64_t nout, int64_t ny, int64_t nx, int r, int depth, int esize, int sms);
 
 // Per-dtype instantiations (one translation unit each).
 int occupancy_stencil_f64(int shape, int r, int depth, const LaunchShape& ls);

@@ -164,7 +164,9 @@ extern "C" int so2dr_run_device_noalloc(int ndim, const int64_t* dims, int radiu
             // (its grid is its tiles)
         } else if (ls.fast && ls.fast != kFastPlane3D) {
             int occ = stencil_occupancy(dtype, shape, radius, depth, ls);
-            if (ls.fast == kFastStar3D) choose_work_split(ls, n0, radius, depth, sms, occ, &a.split);
+            if (ls.fast == kFastStar3D && star_small(ls, n0, ny, nx, radius, depth, (int)esize, sms)) {
+                // (the grid is chosen with the tile)
+            } else if (ls.fast == kFastStar3D) choose_work_split(ls, n0, radius, depth, sms, occ, &a.split);
             else if (ls.fast == kFastBox2D) ls.grid.z = (unsigned)choose_segments((int64_t)ls.grid.x * ls.grid.y, n0, radius, depth, sms, occ, false);
             else choose_row_split(ls, n0, radius, depth, csize, sms, occ, a);
         }

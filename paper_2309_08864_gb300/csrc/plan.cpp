@@ -612,7 +612,7 @@ double kernel_rate_now(const Plan& p, int depth) {
         switch (p.r) {
             case 1: return at({815, 1323, 1494, 1565});
             case 2: return at({703, 885});
-            case 3: return at({528, 376});
+            case 3: return at({606, 376});
             default: return at({494, 258});
         }
     }
@@ -643,7 +643,7 @@ double launch_seconds(const Plan& p, int depth, double planes) {
     if (p.ndim == 3 && p.dtype == SO2DR_F32 && fast_star3d_supported(p.r, depth)) {
         const int sms = 152;
         const int64_t tx = 128 - 2 * ((p.r * depth + 3) / 4 * 4);
-        const int64_t ty = (depth == 1 || p.r >= 3 ? 16 : 32) - 2 * p.r * (depth - 1);
+        const int64_t ty = ((depth == 1 && p.r != 3) || (depth > 1 && p.r >= 3) ? 16 : 32) - 2 * p.r * (depth - 1);
         const int64_t edge = p.r <= 2 ? 1024 : 768;  // the grid the rate was measured on
         const double ovh = 2.0 * p.r * depth + depth;
         const double tiles0 = (double)((edge + tx - 1) / tx) * (double)((edge + ty - 1) / ty);

@@ -238,7 +238,10 @@ int enqueue_stencil(so2dr_plan_s* P, const RunList& rl, const Op& op, cudaStream
         // split the work so that the grid fills the SMs evenly
         int& occ = P->occ_cache[1][o.depth];
         if (!occ) occ = stencil_occupancy(p.dtype, shape, p.r, o.depth, ls);
-        if (ls.fast == kFastStar3D) {
+        if (ls.fast == kFastStar3D && op.host_src < 0 &&
+            star_small(ls, o.dst_hi - o.dst_lo, p.ny, p.nx, p.r, o.depth, (int)p.elem_bytes, P->sm_count)) {
+            // (the grid is chosen with the tile)
+        } else if (ls.fast == kFastStar3D) {
             choose_work_split(ls, o.dst_hi - o.dst_lo, p.r, o.depth, P->sm_count, occ, &a.split);
             // the round split's piece counter: one per stream (the launches
             // of a stream run one after another), beside the status word

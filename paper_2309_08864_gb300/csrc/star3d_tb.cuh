@@ -58,9 +58,15 @@ namespace so2dr {
 // (K * 2R * 16 per thread) and carried cells fit the 255-register limit of a
 // 256-thread CTA; radius 3 and 4 fuse two levels with 2 rows per warp (the
 // 2R = 8 partial sums per cell and level leave no room for more).  One level:
-// 8 warps of 2 rows, two CTAs per SM.
-template <int R, int K> struct StarShape {
-    static constexpr int VY = (K == 1 || R >= 3) ? 2 : 4;
+// 8 warps of 2 rows, two CTAs per SM; radius 3 takes 4 rows and one CTA, whose
+// y neighbours cost half the shared-memory reads (768^3 528 -> 606
+// Gcell-steps/s; radius 2 loses, 702 -> 626, radius 4 is the same).
+// SMALL (radius 1 fused, radius 3 at one level): 2 rows per warp and two CTAs
+// per SM, for grids of so few tiles that a CTA's own pace counts
+// (star_small in kernels.cu).
+template <int R, int K, bool SMALL = false> struct StarShape {
+    static constexpr bool HAS_SMALL = (R == 1 && K > 1) || (R == 3 && K == 1);
+    static constexpr int VY = SMALL ? 2 : R == 3 && K == 1 ? 4 : (K == 1 || R >= 3) ? 2 : 4;
     static constexpr int NW = 8;
     static constexpr int NT = NW * 32;
     static constexpr bool CARRY = K > 1;                // own cells of a level stay in registers
@@ -82,8 +88,8 @@ template <int R, int K> struct StarShape {
     // instruction cache (768^3 in core, unrolled against not: radius 4 376 /
     // 461 at one level, 110 / 245 at two, radius 3 485 / 515 and 329 / 357,
     // 1024^3 radius 2 770 / 859 at two)
-    static constexpr int UNR = R == 1 ? 2 : 1;
-    static constexpr int MINB = K == 1 ? 2 : 1;         // CTAs per SM the registers are sized for
+    static constexpr int UNR = R == 1 && !SMALL ? 2 : 1;
+    static constexpr int MINB = SMALL || (K == 1 && R != 3) ? 2 : 1;         // CTAs per SM the registers are sized for
     // staged columns: 16-bit boxes start on an 8-element boundary (16 bytes),
     // so they carry 8 spare columns and the tile starts 0 or 4 columns in
     template <int ES> static constexpr int lxb() { return ES == 4 ? LX : LX + 8; }
@@ -112,9 +118,9 @@ enum BndMode : int {
     kBndCells = 2,    // boundary rows or fixed planes: per-cell masks
 };
 
-template <typename T, int R, int K, int STG>
+template <typename T, int R, int K, int STG, bool SMALL>
 struct StarTB {
-    using S = StarShape<R, K>;
+    using S = StarShape<R, K, SMALL>;
     static constexpr int VY = S::VY, NW = S::NW, LX = S::LX, LYT = S::LYT, ROWS = S::ROWS, NI = S::NI,
                          PD = S::PD, NB = S::NB, W2 = 2 * R, ES = (int)sizeof(T);
     static constexpr bool ZC = STG == kStageHost, RAG = STG == kStageRagged;
@@ -475,7 +481,11 @@ struct StarTB {
         // a fixed plane among their targets (z' - R .. z') needs the cell path
         const bool all = p >= ps_lo && p < ps_hi;
         const bool fixed = za + p - (K - 1) * (R + 1) < 2 * R || za + p >= n0 - R;
-        if constexpr (R == 1) {
+        if constexpr (SMALL && R == 1) {
+            // one body for every phase: a short launch pays for each
+            // instruction it fetches
+            levels<K - 1, PH, kBndCells, false>(p, all);
+        } else if constexpr (R == 1) {
             // short bodies: straight-line phases for the steady state, and
             // the checked ones for head, tail and fixed planes
             if (all && !fixed && wmode == kBndNone) levels<K - 1, PH, kBndNone, true>(p, true);
@@ -750,11 +760,11 @@ struct StarTB {
 
 // One instantiation per staging mode, so that the launches of the copy-engine
 // pipeline on aligned rows carry none of the others' code
-template <typename T, int R, int K, int STG = kStageTma>
-__global__ void __launch_bounds__(StarShape<R, K>::NT, STG == kStageRagged && R > 2 ? 1 : StarShape<R, K>::MINB)
+template <typename T, int R, int K, int STG = kStageTma, bool SMALL = false>
+__global__ void __launch_bounds__(StarShape<R, K>::NT, STG == kStageRagged && (R > 2 || SMALL) ? 1 : StarShape<R, K, SMALL>::MINB)
     star3d_tb_kernel(const StencilArgs a, const __grid_constant__ CUtensorMap tmap) {
     extern __shared__ __align__(1024) unsigned char smem_tb[];
-    StarTB<T, R, K, STG> k(a, &tmap);
+    StarTB<T, R, K, STG, SMALL> k(a, &tmap);
     k.run(smem_tb);
 }
 
