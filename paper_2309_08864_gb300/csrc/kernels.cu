@@ -157,6 +157,10 @@ LaunchShape stencil_launch_shape(int shape, int r, int depth, int64_t n0, int64_
             case 66: fast_shape<4, 2>(ls, ny, nx, esize); break;
         }
         if (ls.ok) return ls;
+        // more rows than the star kernel's grid reaches (65535 tiles in y): all
+        // of the choice is taken back, the generic kernel has its own geometry
+        ls.fast = 0;
+        ls.ragged = false;
     }
     int H = r * depth;
     // (only depths the generic kernel takes too, so that the deepest supported

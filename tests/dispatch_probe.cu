@@ -1,0 +1,23 @@
+// dispatch_probe.cu -- the library's own choice of kernel and geometry for one
+// launch, for tests (host code only: no CUDA call).
+#include "kernels.hpp"
+
+using namespace so2dr;
+
+// out: {ok, kernel family, 2-row tile, ragged, grid x, y, z, tile x, y, shared
+// bytes, split, split2, split_at}; the families are LaunchShape::fast's.
+extern "C" void probe_launch(int dtype, int shape, int r, int depth, int64_t n0, int64_t ny, int64_t nx, int64_t nout,
+                             int sms, int occ, int64_t* out) {
+    const int csize = dtype == SO2DR_F64 ? 8 : 4;
+    const int esize = dtype == SO2DR_F64 ? 8 : dtype == SO2DR_F32 ? 4 : 2;
+    LaunchShape ls = stencil_launch_shape(shape, r, depth, n0, ny, nx, csize, esize);
+    StencilArgs a = {};
+    a.split_at = nout;
+    if (ls.ok && ls.fast == kFastRow2D && !tile2d_short(ls, shape, nout, nx, r, depth, csize, sms))
+        choose_row_split(ls, nout, r, depth, csize, sms, occ, a);
+    if (ls.ok && ls.fast == kFastStar3D) star_small(ls, nout, ny, nx, r, depth, esize, sms);
+    const int64_t v[13] = {ls.ok, ls.fast, ls.small, ls.ragged, ls.ok ? ls.grid.x : 0, ls.ok ? ls.grid.y : 0,
+                           ls.ok ? ls.grid.z : 0, ls.ok ? ls.tx : 0, ls.ok ? ls.ty : 0, ls.ok ? (int64_t)ls.smem : 0,
+                           a.split, a.split2, a.split_at};
+    for (int i = 0; i < 13; ++i) out[i] = v[i];
+}
