@@ -194,6 +194,11 @@ LaunchShape stencil_launch_shape(int shape, int r, int depth, int64_t n0, int64_
     return ls;
 }
 
+bool star3d_reads_host(int r, int depth, int64_t n0, int64_t ny, int64_t nx, int esize) {
+    const LaunchShape ls = stencil_launch_shape(kStar3D, r, depth, n0, ny, nx, 4, esize);
+    return ls.ok && ls.fast == kFastStar3D && !ls.ragged;
+}
+
 int stencil_max_depth(int shape, int r, int csize) {
     int best = 0;
     for (int d = 1; d <= 16; ++d) {

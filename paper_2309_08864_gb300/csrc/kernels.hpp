@@ -50,6 +50,10 @@ bool wide_box2d(int r, int depth, int64_t nx, int csize);
 // (R, K) pairs the 2D kernel is instantiated for (shape kBox2D or kStar2D).
 bool row2d_supported(int shape, int r, int depth, int csize);
 
+// Whether a 3D star launch of FP32 arithmetic goes to the star kernel with its
+// TMA staging, the one that can also read mapped host planes.
+bool star3d_reads_host(int r, int depth, int64_t n0, int64_t ny, int64_t nx, int esize);
+
 // csize: compute-type bytes; esize: storage-type bytes.
 LaunchShape stencil_launch_shape(int shape, int r, int depth, int64_t n0, int64_t ny, int64_t nx, int csize, int esize);
 

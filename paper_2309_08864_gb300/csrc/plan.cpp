@@ -11,7 +11,7 @@ namespace so2dr {
 
 bool fast_star3d_supported(int r, int depth);
 int choose_segments(int64_t tiles, int64_t nout, int r, int depth, int sms, int occ, bool share_sm);
-bool fast_star3d_row_ok(int64_t nx, int esize);
+bool star3d_reads_host(int r, int depth, int64_t n0, int64_t ny, int64_t nx, int esize);
 
 
 int64_t elem_size(int dtype) {
@@ -897,14 +897,14 @@ int build_plan(Plan& p, int ndim, const int64_t* dims, int radius, int kind, con
     if (p.kind != SO2DR_VARCOEF_STAR && p.rounds > 0)
         if (!build_result_reuse(p, p.rr, p.budget, &p.rr_chunks)) p.rr_chunks = 0;
     // zero-copy input: the first launch of every chunk must run the 3D star
-    // kernel (the one that can read mapped host planes)
+    // kernel (the one that can read mapped host planes), which the dispatch
+    // itself says: another kernel would read planes nobody filled
     p.zc_ok = false;
-    if (p.kind == SO2DR_STAR && p.ndim == 3 && p.dtype != SO2DR_F64 && p.rounds > 0 &&
-        fast_star3d_row_ok(p.nx, (int)p.elem_bytes) && !std::getenv("SO2DR_GENERIC_KERNEL")) {
+    if (p.kind == SO2DR_STAR && p.ndim == 3 && p.dtype != SO2DR_F64 && p.rounds > 0) {
         bool all_fast = true;
         for (int t = 0; t < p.rounds; ++t) {
             const int kk = round_steps(p.T, p.k_off, t);
-            all_fast = all_fast && fast_star3d_supported(p.r, std::min(kk, p.k_on));
+            all_fast = all_fast && star3d_reads_host(p.r, std::min(kk, p.k_on), p.n0, p.ny, p.nx, (int)p.elem_bytes);
         }
         ForwardOpts zo;
         zo.zero_copy = true;

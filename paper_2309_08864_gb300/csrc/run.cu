@@ -220,7 +220,11 @@ int enqueue_stencil(so2dr_plan_s* P, const RunList& rl, const Op& op, cudaStream
     a.ty = ls.ty;
     a.status = reinterpret_cast<int*>(P->arena + rl.arena_bytes - kAlign);  // the run list's status word
     if (op.host_src >= 0) {
-        // zero-copy input: the device mapping of the host array
+        // zero-copy input: the device mapping of the host array.  Only the star
+        // kernel's TMA form reads it (SO2DR_GENERIC_KERNEL set after planning
+        // sends the launch elsewhere)
+        if (ls.fast != kFastStar3D || ls.ragged)
+            return set_error(SO2DR_E_DEVICE_CHECK, "zero-copy launch on a kernel that cannot read the host grid");
         if (op.host_src >= (int)P->host_dev.size() || !P->host_dev[op.host_src])
             return set_error(SO2DR_E_DEVICE_CHECK, "zero-copy launch without a mapped host grid");
         a.host_in = P->host_dev[op.host_src];

@@ -1,6 +1,8 @@
 """The choice of kernel and launch geometry (host only, no GPU)."""
+import numpy as np
 import pytest
 
+from paper_2309_08864_gb300 import so2dr
 from tests import dispatch
 
 RK = [(1, 1), (1, 2), (1, 3), (1, 4), (2, 1), (2, 2), (3, 1), (3, 2), (4, 1), (4, 2)]
@@ -21,3 +23,24 @@ def test_star_kernel_and_its_geometry_go_together(r, k, dtype, nx):
     over = dispatch.launch(dtype, "star", r, k, (200, limit + 1, nx))
     assert not over["ok"] or over["fast"] == dispatch.GENERIC
     assert not over["ok"] or over["gy"] * over["ty"] > limit
+
+
+@pytest.mark.parametrize("dtype,r,k", [("f32", 1, 4), ("f32", 4, 1), ("bf16", 1, 3)])
+def test_zero_copy_only_where_the_star_kernel_runs(dtype, r, k):
+    """The mapped host planes are read by the star kernel alone: plans whose
+    launches its grid or its 32-bit indices cannot take have no zero-copy form
+    (the generic kernel would read planes that nobody filled)."""
+    c = np.full(1 + 6 * r, 1.0 / (1 + 6 * r))
+
+    def zc(*dims):
+        p = so2dr.Plan(dims, r, "star", c, k, min_chunks=2, k_on=k, k_off=k, budget_bytes=0, dtype=dtype)
+        n, runs_on = p.info["zero_copy"], dispatch.launch(dtype, "star", r, k, dims)
+        p.close()
+        return n, runs_on["fast"] == dispatch.STAR3D and not runs_on["ragged"]
+
+    rows = 65535 * dispatch.launch(dtype, "star", r, k, (64, 4096, 24))["ty"]
+    for dims in [(64, 40, 24), (64, 40, 20), (64, 40, 21), (64, rows, 24), (64, rows + 1, 24), (64, 9, 1 << 30),
+                 (64, 9, (1 << 30) + 8)]:
+        has, runs_on = zc(*dims)
+        assert has == runs_on, dims
+    assert zc(64, 40, 24)[0] and not zc(64, rows + 1, 24)[0] and not zc(64, 9, (1 << 30) + 8)[0]

@@ -70,3 +70,21 @@ def test_zero_copy_work_splits(dims, r, kon, koff, dtype, split, monkeypatch):
     plan.run(ic, in_core=True)
     plan.close()
     assert torch.equal(zc.view(torch.uint8), ic.view(torch.uint8)), "zero-copy != in-core"
+
+
+def test_zero_copy_plan_refuses_the_generic_kernel(monkeypatch):
+    """A zero-copy plan whose launches are sent to the generic kernel after
+    planning is refused: that kernel does not read the host grid."""
+    dims = (72, 70, 132)
+    plan = so2dr.Plan(dims, 1, "star", [0.4] + [0.1] * 6, 8, min_chunks=3, k_on=4, k_off=8, budget_bytes=0, dtype="f32")
+    u = gu.pinned_from_storage(inputs.to_storage(inputs.draw_box(1, dims), so2dr.F32), so2dr.F32)
+    before = u.clone()
+    monkeypatch.setenv("SO2DR_GENERIC_KERNEL", "1")
+    with pytest.raises(so2dr.So2drError) as e:
+        plan.run(u, in_core=3)
+    assert e.value.code == so2dr.E_DEVICE_CHECK
+    assert (u == before).all()
+    monkeypatch.delenv("SO2DR_GENERIC_KERNEL")
+    plan.run(u, in_core=3)
+    assert not (u == before).all()
+    plan.close()
