@@ -367,14 +367,22 @@ void choose_row_split(LaunchShape& ls, int64_t nout, int r, int depth, int csize
 bool tile2d_short(LaunchShape& ls, int shape, int64_t nout, int64_t nx, int r, int depth, int csize, int sms) {
     // Rows of 32 columns per SM up to which the tile is the faster one
     // (in-core Gcell-steps/s, strips / tile).  FP64, fused: 80x512 radius 1, 4
-    // levels 5.6 / 15.7, 512^2 28 / 43, 1024^2 60 / 73 (215 rows per SM); one
-    // level has little halo to save (512^2 20.9 / 20.3).  FP32: 81-point box,
+    // levels 5.6 / 15.7, 512^2 28 / 43, 1024^2 60 / 73 (215 rows per SM).
+    // FP64, wide halos: a segment streams more halo than rows of its own (us a
+    // launch, strips / tile / generic kernel).  One level, radius 2 star
+    // 64x1000 14.5 / 8.7 / 13.4, 300x12800 (789 rows) 133 / 77 / 146; 25-point
+    // box 250x6000 102 / 104 / 142, 300x12800 357 / 226 / 281; radius 4 star
+    // 75x3882 43 / 21 / 35, 300x12800 264 / 133 / 207; 81-point box 250x6000
+    // 357 / 293 / 314, 2000^2 (829 rows) 807 / 698 / 910.  Two levels, 81-point
+    // box 500x6000 (618 rows) 1255 / 1155 / 1233, 2000^2 1578 / 1623 / 1798;
+    // 49-point box 1000x3882 (802 rows) 872 / 946 / 1072.  Radius 1 at one
+    // level has little halo to save (512^2 20.9 / 20.3 Gcell-steps/s).  FP32: 81-point box,
     // one level 512^2 14.0 / 18.8, 1024^2 49 / 52; radius 3, 4 levels,
     // 701x1003 93 / 106; 9-point box, 8 levels 512^2 74 / 85 (54 rows), 1024^2
     // 272 / 219; radius 1, 4 levels 80x512 18 / 20, 256^2 (13 rows) 26 / 25,
     // 512^2 94 / 72.
     const int H = r * depth;
-    const int64_t limit = csize == 8 ? (depth > 1 ? 256 : 0)
+    const int64_t limit = csize == 8 ? (depth == 1 ? (r > 1 ? 1024 : 0) : r > 2 ? 640 : 256)
                           : (shape == kBox2D && r >= 3) || H >= 12 ? 160
                           : H >= 6 ? 60 : depth > 1 ? 12 : 0;
     const int64_t gx = (nx + kTileX - 1) / kTileX;

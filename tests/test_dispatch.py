@@ -44,3 +44,13 @@ def test_zero_copy_only_where_the_star_kernel_runs(dtype, r, k):
         has, runs_on = zc(*dims)
         assert has == runs_on, dims
     assert zc(64, 40, 24)[0] and not zc(64, rows + 1, 24)[0] and not zc(64, 9, (1 << 30) + 8)[0]
+
+
+@pytest.mark.parametrize("kind,r,k", [(kind, r, 1) for kind in ("star", "box") for r in (2, 3, 4)] + [("box", 4, 2), ("star", 3, 2)])
+def test_short_fp64_launches_take_the_tile(kind, r, k):
+    """Chunk launches of wide halos in FP64: the strips' segments stream
+    mostly halo there and were slower than the generic kernel."""
+    for dims, nout in [((599, 3882), 75), ((140, 2112), 140), ((64, 1000), 64), ((20, 3882), 20), ((250, 6000), 250),
+                       ((12800, 12800), 300 if k == 1 else 200)]:
+        assert dispatch.launch("f64", kind, r, k, dims, nout)["fast"] == dispatch.TILE2D
+    assert dispatch.launch("f64", kind, r, k, (12800, 12800))["fast"] == dispatch.ROW2D

@@ -53,8 +53,8 @@ def _same_bytes(dims, kind, r, k, name, modes, monkeypatch):
         assert torch.equal(t, runs[-1]), "mode %d differs from the generic kernel" % m
 
 
-@pytest.mark.parametrize("dims", [(39100, 20), (39100, 29), (9900, 124), (9900, 125), (7900, 149), (3100, 411),
-                                  (17, 73700), (17, 73701)])
+@pytest.mark.parametrize("dims", [(156000, 20), (156000, 29), (39000, 124), (39000, 125), (31300, 149), (12100, 411),
+                                  (17, 294000), (17, 294001)])
 @pytest.mark.parametrize("kind,r,k,name", CASES)
 def test_strips_match_generic_kernel_bitwise(kind, r, k, name, dims, monkeypatch):
     sh = dispatch.launch(name, kind, r, k, dims, sms=_sms())
@@ -73,3 +73,10 @@ def test_long_and_short_segments_match_generic_kernel_bitwise(kind, r, k, name, 
         sh = dispatch.launch(name, kind, r, k, dims, sms=_sms(), occ=occ)
         assert sh["fast"] == dispatch.ROW2D and sh["split2"] > 0 and 0 < sh["split_at"] < dims[0]
     _same_bytes(dims, kind, r, k, name, (1, 0), monkeypatch)
+
+
+@pytest.mark.parametrize("dims", [(75, 3882), (64, 1000), (33, 125), (20, 31)])
+@pytest.mark.parametrize("kind,r,k", [(kind, r, 1) for kind in ("star", "box") for r in (2, 3, 4)] + [("box", 4, 2), ("star", 3, 2)])
+def test_fp64_tile_of_wide_halos_matches_generic_kernel_bitwise(kind, r, k, dims, monkeypatch):
+    assert dispatch.launch("f64", kind, r, k, dims, sms=_sms())["fast"] == dispatch.TILE2D
+    _same_bytes(dims, kind, r, k, "f64", (1, 0), monkeypatch)
