@@ -293,10 +293,10 @@ void choose_work_split(LaunchShape& ls, int64_t nout, int r, int depth, int sms,
     }
 }
 
-// Launches of up to this many cells take the 2-row tile (radius 1 fused, radius
-// 3 at one level).  In-core Gcell-steps/s, 4 rows / 2 rows: four levels 48x80x132
-// 89 / 96, 64^3 50 / 56, 101x99x97 117 / 151, 96^3 153 / 155, 128^3 252 / 186,
-// 160^3 two levels 329 / 298; radius 3 64^3 18.3 / 21.3, 128^3 111 / 99.
+// Launches of up to this many cells may take the 2-row tile (radius 1 fused,
+// radius 3 at one level).  In-core Gcell-steps/s, 4 rows / 2 rows: four levels
+// 48x80x132 89 / 96, 64^3 50 / 56, 96^3 153 / 155, 128^3 252 / 186, 160^3 two
+// levels 329 / 298; radius 3 64^3 18.3 / 21.3, 128^3 111 / 99.
 constexpr double kSmallCells = 1e6;
 
 bool star_small(LaunchShape& ls, int64_t nout, int64_t ny, int64_t nx, int r, int depth, int esize, int sms) {
@@ -320,6 +320,21 @@ bool star_small(LaunchShape& ls, int64_t nout, int64_t ny, int64_t nx, int r, in
         const int64_t c = (tiles * n + sms - 1) / sms;
         const double cost = ((double)((nout + n - 1) / n) + ovh) * (3.6 * (double)(c / 2) + 2.2 * (double)(c % 2));
         if (!best_n || cost < best * 0.98) { best_n = n; best = cost; }
+    }
+    // Its planes are quicker (a 4-row CTA's plane takes 1.29 times as long at
+    // three and four levels, 1.4 times at the others), but it cuts a plane into
+    // more tiles and so the planes into fewer, longer segments; and on a long
+    // segment the 4-row kernel's straight-line phases win.  Us a launch, 4 rows
+    // / 2 rows: three levels 120x129x16 16.4 / 18.5, 24x512x24 15.0 / 16.4,
+    // 64^3 16.2 / 14.5, 600x40x24 22.5 / 24.6; four levels 185x154x16 30.7 /
+    // 36.9, 300x48x48 23.9 / 24.6; two levels 2000x20x24 22.5 / 28.7, 60x200x32
+    // 13.5 / 12.8; radius 3 185x154x16 16.4 / 18.4.  (Ragged rows: the 2-row
+    // tile, three levels 140x200x33 34.8 / 32.8.)
+    if (!ls.ragged) {
+        const int64_t t4 = (int64_t)ls.grid.x * ls.grid.y;
+        const int n4 = choose_segments(t4, nout, r, depth, sms, 1, true);
+        const double cost4 = (double)((t4 * n4 + sms - 1) / sms) * ((double)((nout + n4 - 1) / n4) + ovh);
+        if (best > cost4 * 2.2 * (r == 1 && depth > 2 ? 1.29 : 1.4) || nout > (12 + depth) * (int64_t)best_n) return false;
     }
     t.grid.z = (unsigned)best_n;
     ls = t;

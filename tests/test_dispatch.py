@@ -54,3 +54,14 @@ def test_short_fp64_launches_take_the_tile(kind, r, k):
                        ((12800, 12800), 300 if k == 1 else 200)]:
         assert dispatch.launch("f64", kind, r, k, dims, nout)["fast"] == dispatch.TILE2D
     assert dispatch.launch("f64", kind, r, k, (12800, 12800))["fast"] == dispatch.ROW2D
+
+
+@pytest.mark.parametrize("dims,r,k,small", [
+    ((120, 129, 16), 1, 3, 0), ((185, 154, 16), 1, 4, 0), ((24, 512, 24), 1, 3, 0), ((2000, 20, 24), 1, 2, 0),
+    ((600, 40, 24), 1, 3, 0), ((185, 154, 16), 3, 1, 0), ((128, 128, 128), 1, 4, 0),
+    ((48, 80, 132), 1, 4, 1), ((64, 64, 64), 1, 4, 1), ((64, 64, 64), 1, 2, 1), ((60, 200, 32), 1, 2, 1),
+    ((6, 352, 400), 1, 4, 1), ((64, 64, 64), 3, 1, 1), ((140, 200, 33), 1, 3, 1)])
+def test_two_row_tile_only_where_its_segments_stay_short(dims, r, k, small):
+    """The 2-row tile cuts a plane into more tiles and so the planes into
+    fewer segments: narrow rows and long grids are the 4-row tile's."""
+    assert dispatch.launch("f32", "star", r, k, dims)["small"] == small

@@ -32,8 +32,8 @@ def _same_bytes(dims, r, k, name, modes, monkeypatch):
         assert torch.equal(t, runs[-1]), "mode %d differs from the generic kernel" % m
 
 
-# odd rows, rows of even length that are no whole vectors, aligned rows
-@pytest.mark.parametrize("dims", [(70, 121, 125), (41, 190, 134), (41, 97, 264)])
+# odd rows, rows of even length that are no whole vectors, aligned rows; a long grid of narrow rows
+@pytest.mark.parametrize("dims", [(70, 121, 125), (41, 190, 134), (41, 97, 264), (2000, 20, 24)])
 @pytest.mark.parametrize("r,k,name", CASES)
 def test_large_launches_match_generic_kernel_bitwise(r, k, name, dims, monkeypatch):
     sh = dispatch.launch(name, "star", r, k, dims)
