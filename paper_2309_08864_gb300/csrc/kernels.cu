@@ -6,6 +6,7 @@
 #include "star3d_tb.cuh"
 #include "tile2d_tb.cuh"
 
+#include <algorithm>
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
@@ -70,10 +71,16 @@ void row_shape(LaunchShape& ls, int shape, int r, int depth, int64_t nx, int csi
 
 // The plane kernel's tile: the one that computes the fewest rows of 32 cells
 // over the grid (halos and the grid's last, partial tiles included; a row
-// loaded counts 0.3, a phase's barrier and bookkeeping 12).
-void plane_shape(LaunchShape& ls, int r, int depth, int64_t ny, int64_t nx, int csize) {
+// loaded counts 0.3, a phase's barrier and bookkeeping 12).  With sms > 0, for
+// one launch of nout planes that cannot fill the device with such tiles: the
+// least time of the busiest SM instead.  A CTA of a segment of len planes loads
+// one plane a phase, len + 2H + depth phases that last 32 rows' time at least,
+// and level l computes len + 2r(depth - l) planes; the given tile keeps its
+// place unless another is 10% better.
+void plane_shape(LaunchShape& ls, int r, int depth, int64_t ny, int64_t nx, int csize, int64_t nout = 0, int sms = 0) {
     const int H = r * depth;
-    double best = 0;
+    const int lx0 = ls.lx, ly0 = ls.ly;
+    double best = -1;
     for (int lx : {32, 64})
         for (int ly = 2 * H + 4; ly <= kPlaneMaxRows * (kPlaneThreads / lx); ly += 4) {
             const int tx = lx - 2 * H, ty = ly - 2 * H;
@@ -81,10 +88,21 @@ void plane_shape(LaunchShape& ls, int r, int depth, int64_t ny, int64_t nx, int 
             if (tx <= 0 || smem > kSmemLimit) continue;
             const int64_t gx = (nx + tx - 1) / tx, gy = (ny + ty - 1) / ty;
             if (gx > 2147483647 || gy > 65535) continue;
-            double rows = 0.3 * ly;
-            for (int l = 1; l <= depth; ++l) rows += ly - 2 * l * r;
-            const double cost = (double)gx * (double)gy * (rows * (lx / 32) + 12.0);
-            if (ls.ok && cost >= best) continue;
+            double cost;
+            if (sms > 0) {
+                const int64_t tiles = gx * gy, fill = tiles < sms ? sms / tiles : 1;
+                const int64_t n = std::min<int64_t>(std::min<int64_t>(fill, 64), nout);
+                const double len = (double)nout / (double)n, phases = len + 2.0 * H + depth;
+                double rows = phases * 0.3 * ly;
+                for (int l = 1; l <= depth; ++l) rows += (len + 2.0 * r * (depth - l)) * (ly - 2 * l * r);
+                cost = (double)((tiles * n + sms - 1) / sms) * (rows * (lx / 32) + phases * 32.0);
+                if (lx == lx0 && ly == ly0) cost *= 0.9;
+            } else {
+                double rows = 0.3 * ly;
+                for (int l = 1; l <= depth; ++l) rows += ly - 2 * l * r;
+                cost = (double)gx * (double)gy * (rows * (lx / 32) + 12.0);
+            }
+            if (best >= 0 && cost >= best) continue;
             best = cost;
             ls.lx = lx;
             ls.ly = ly;
@@ -291,6 +309,21 @@ void choose_work_split(LaunchShape& ls, int64_t nout, int r, int depth, int sms,
     } else {
         ls.grid.z = (unsigned)nseg;
     }
+}
+
+// FP64 launches of up to this many cells get a tile of their own.  Us a launch,
+// the grid's tile / this one / generic kernel: variable coefficients, two levels
+// 38x39x32 57.9 / 25.2 / 40.9, 4x256x256 60 / 35 / 39, 20x256x256 142 / 121 /
+// 135, four levels 8x256x256 165 / 115 / 147; radius 1 48^3 one level 20.9 /
+// 12.3 / 18.9, radius 2 48^3 31.3 / 15.4 / 25.3, 10x512x512 94 / 64 / 88.
+// Larger ones keep the grid's tile (64x512x512 radius 4 1106 / 1181 / 1450), and
+// so does FP32, whose rows cost little beside a phase (variable coefficients
+// 64^3 one level 12.5 / 16.4 / 27.2).
+constexpr double kPlaneFitCells = 3e6;
+
+void plane_fit(LaunchShape& ls, int64_t nout, int r, int depth, int64_t ny, int64_t nx, int csize, int sms) {
+    if (csize != 8 || sms <= 0 || nout <= 0 || (double)nout * (double)ny * (double)nx > kPlaneFitCells) return;
+    plane_shape(ls, r, depth, ny, nx, csize, nout, sms);
 }
 
 // Launches of up to this many cells may take the 2-row tile (radius 1 fused,

@@ -96,6 +96,10 @@ void choose_row_split(LaunchShape& ls, int64_t nout, int r, int depth, int csize
 // is rated faster; false: keep ls.
 bool tile2d_short(LaunchShape& ls, int shape, int64_t nout, int64_t nx, int r, int depth, int csize, int sms);
 
+// Gives a small FP64 launch of the plane kernel a tile that fills the device
+// (sets ls; its segments are chosen afterwards as for any other tile).
+void plane_fit(LaunchShape& ls, int64_t nout, int r, int depth, int64_t ny, int64_t nx, int csize, int sms);
+
 // 3D star kernel (star3d_tb.cuh), a translation unit per storage type and
 // kind of rows.
 int occupancy_star3d_f32(int r, int depth, const LaunchShape& ls);

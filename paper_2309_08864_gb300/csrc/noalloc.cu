@@ -160,6 +160,7 @@ extern "C" int so2dr_run_device_noalloc(int ndim, const int64_t* dims, int radiu
         StencilArgs a;
         std::memset(&a, 0, sizeof(a));
         if (ls.fast == kFastRow2D) tile2d_short(ls, shape, n0, nx, radius, depth, csize, sms);
+        if (ls.fast == kFastPlane3D) plane_fit(ls, n0, radius, depth, ny, nx, csize, sms);
         if (ls.fast == kFastTile2D) {
             // (its grid is its tiles)
         } else if (ls.fast && ls.fast != kFastPlane3D) {

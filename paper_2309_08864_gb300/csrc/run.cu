@@ -190,6 +190,7 @@ int enqueue_stencil(so2dr_plan_s* P, const RunList& rl, const Op& op, cudaStream
     if (o.src_hi - o.src_lo > bi.cap || o.dst_slot0 < 0 || o.dst_slot0 + (o.dst_hi - o.dst_lo) > bo.cap)
         return set_error(SO2DR_E_DEVICE_CHECK, "kernel op exceeds its buffer");
     if (ls.fast == kFastRow2D) tile2d_short(ls, shape, o.dst_hi - o.dst_lo, p.nx, p.r, o.depth, csize, P->sm_count);
+    if (ls.fast == kFastPlane3D) plane_fit(ls, o.dst_hi - o.dst_lo, p.r, o.depth, p.ny, p.nx, csize, P->sm_count);
     StencilArgs a;
     std::memset(&a, 0, sizeof(a));
     a.in = P->arena + bi.offset;

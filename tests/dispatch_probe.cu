@@ -15,6 +15,10 @@ extern "C" void probe_launch(int dtype, int shape, int r, int depth, int64_t n0,
     a.split_at = nout;
     if (ls.ok && ls.fast == kFastRow2D && !tile2d_short(ls, shape, nout, nx, r, depth, csize, sms))
         choose_row_split(ls, nout, r, depth, csize, sms, occ, a);
+    if (ls.ok && ls.fast == kFastPlane3D) {
+        plane_fit(ls, nout, r, depth, ny, nx, csize, sms);
+        ls.grid.z = (unsigned)choose_segments((int64_t)ls.grid.x * ls.grid.y, nout, r, depth, sms, 1, false);
+    }
     if (ls.ok && ls.fast == kFastStar3D) star_small(ls, nout, ny, nx, r, depth, esize, sms);
     const int64_t v[13] = {ls.ok, ls.fast, ls.small, ls.ragged, ls.ok ? ls.grid.x : 0, ls.ok ? ls.grid.y : 0,
                            ls.ok ? ls.grid.z : 0, ls.ok ? ls.tx : 0, ls.ok ? ls.ty : 0, ls.ok ? (int64_t)ls.smem : 0,

@@ -65,3 +65,20 @@ def test_two_row_tile_only_where_its_segments_stay_short(dims, r, k, small):
     """The 2-row tile cuts a plane into more tiles and so the planes into
     fewer segments: narrow rows and long grids are the 4-row tile's."""
     assert dispatch.launch("f32", "star", r, k, dims)["small"] == small
+
+
+@pytest.mark.parametrize("kind,r,k,dims", [("varcoef", 1, 2, (38, 39, 32)), ("varcoef", 1, 2, (4, 256, 256)),
+                                           ("varcoef", 1, 4, (8, 256, 256)), ("star", 1, 1, (48, 48, 48)),
+                                           ("star", 2, 1, (10, 512, 512)), ("star", 2, 2, (48, 48, 48)),
+                                           ("star", 4, 1, (48, 48, 48))])
+def test_small_fp64_plane_launches_fill_the_device(kind, r, k, dims):
+    """A launch too small to occupy the SMs with the tile of least halo (38 x
+    39 x 32, two levels: one tile, a few segments) gets smaller tiles; the
+    tile still covers the grid and fits the shared memory."""
+    sh = dispatch.launch("f64", kind, r, k, dims)
+    large = dispatch.launch("f64", kind, r, k, (4000,) + dims[1:])  # the grid's tile
+    assert sh["fast"] == large["fast"] == dispatch.PLANE3D
+    assert sh["tx"] * sh["ty"] < large["tx"] * large["ty"]
+    assert sh["gx"] * sh["tx"] >= dims[2] and sh["gy"] * sh["ty"] >= dims[1] and sh["smem"] <= 227 << 10
+    assert 1 <= sh["gz"] <= dims[0]
+    assert dispatch.launch("f32", "varcoef", 1, 2, dims)["tx"] == dispatch.launch("f32", "varcoef", 1, 2, (4000,) + dims[1:])["tx"]

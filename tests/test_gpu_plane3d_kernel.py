@@ -6,6 +6,7 @@ import numpy as np
 import pytest
 
 from paper_2309_08864_gb300 import inputs, so2dr
+from tests import dispatch
 from tests import gpu_util as gu
 from tests.test_gpu_parity import _coeffs
 
@@ -18,6 +19,21 @@ pytestmark = pytest.mark.gpu
                                            ("varcoef", 1, 1, "f32"), ("varcoef", 1, 4, "f32"),
                                            ("varcoef", 1, 6, "f32"), ("varcoef", 1, 3, "f64")])
 def test_plane_kernel_matches_generic_kernel_bitwise(kind, r, k, name, dims, monkeypatch):
+    _same_bytes(kind, r, k, name, dims, monkeypatch)
+
+
+# the tile of a large FP64 launch, and ones fitted to few and to thin planes
+@pytest.mark.parametrize("dims", [(61, 230, 231), (13, 301, 257), (70, 40, 61)])
+@pytest.mark.parametrize("kind,r,k", [("star", 1, 4), ("star", 2, 2), ("star", 4, 1), ("varcoef", 1, 3)])
+def test_large_and_fitted_fp64_tiles_match_generic_kernel_bitwise(kind, r, k, dims, monkeypatch):
+    grid_tile = dispatch.launch("f64", kind, r, k, (4000,) + dims[1:])
+    own = dispatch.launch("f64", kind, r, k, dims)
+    if dims[0] == 61:
+        assert (own["tx"], own["ty"]) == (grid_tile["tx"], grid_tile["ty"])
+    _same_bytes(kind, r, k, "f64", dims, monkeypatch)
+
+
+def _same_bytes(kind, r, k, name, dims, monkeypatch):
     import torch
     dtype = so2dr.DTYPES[name]
     st = inputs.to_storage(inputs.draw_box(3, dims), dtype)
