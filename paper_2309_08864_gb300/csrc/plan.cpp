@@ -797,11 +797,11 @@ int build_plan(Plan& p, int ndim, const int64_t* dims, int radius, int kind, con
         p.d = std::min<int64_t>(min_chunks, p.n0 - 2 * p.r);
         partition_planes(p);
     } else {
-        std::vector<int> kons, koffs;
+        std::vector<int> kons, deeper, koffs;
         if (k_on) kons.push_back(k_on);
         else
             for (int v : {1, 2, 3, 4, 5, 6, 7, 8, 10, 12, 16})
-                if (v <= p.max_kon && v <= p.max_kon_auto) kons.push_back(v);
+                if (v <= p.max_kon) (v <= p.max_kon_auto ? kons : deeper).push_back(v);
         if (k_off) koffs.push_back(k_off);
         else {
             for (int64_t v = 1; v <= std::min<int64_t>(T, 64); ++v) koffs.push_back((int)v);
@@ -822,31 +822,34 @@ int build_plan(Plan& p, int ndim, const int64_t* dims, int radius, int kind, con
             for (int no : {2, 1})
                 if ((fla < 0 || fla == la) && (fno < 0 || fno == no)) opts.push_back({la, no});
         if (opts.empty()) opts.push_back({1, 2});
-        for (int ko : koffs) {
-            for (int kn : kons) {
-                if (kn > ko && koffs.size() > 1) continue;
-                for (auto [la, no] : opts) {
-                    Plan q = p;
-                    q.k_off = ko;
-                    q.k_on = std::min(kn, ko);
-                    q.rounds = (int)((T + ko - 1) / ko);
-                    q.lookahead = la;
-                    q.n_out = no;
-                    int d = fit_chunks(q, min_chunks);
-                    if (!d) continue;
-                    double ms = predict_ms(q);
-                    Candidate c;
-                    c.k_off = q.k_off;
-                    c.k_on = q.k_on;
-                    c.d = d;
-                    c.lookahead = la;
-                    c.n_out = no;
-                    c.predicted_ms = ms;
-                    feasible.push_back(c);
-                    if (search && search->ranked) search->ranked->push_back(c);
-                    if (ms < best) best = ms;
-                }
+        auto consider = [&](int ko, int kn) {
+            for (auto [la, no] : opts) {
+                Plan q = p;
+                q.k_off = ko;
+                q.k_on = std::min(kn, ko);
+                q.rounds = (int)((T + ko - 1) / ko);
+                q.lookahead = la;
+                q.n_out = no;
+                int d = fit_chunks(q, min_chunks);
+                if (!d) continue;
+                double ms = predict_ms(q);
+                Candidate c;
+                c.k_off = q.k_off;
+                c.k_on = q.k_on;
+                c.d = d;
+                c.lookahead = la;
+                c.n_out = no;
+                c.predicted_ms = ms;
+                feasible.push_back(c);
+                if (search && search->ranked) search->ranked->push_back(c);
+                if (ms < best) best = ms;
             }
+        };
+        for (const std::vector<int>* depths : {&kons, &deeper}) {
+            if (depths == &deeper && !(feasible.empty() && p.deeper_if_infeasible)) break;
+            for (int ko : koffs)
+                for (int kn : *depths)
+                    if (kn <= ko || koffs.size() == 1) consider(ko, kn);
         }
         // Among the candidates predicted within 2% of the best, take the ones
         // with the fewest rounds (least host-link traffic); among those

@@ -110,6 +110,7 @@ struct Plan {
     int lookahead = 1;                // circular buffer holds the next chunk's new planes too (1) or not (0)
     int n_out = 2;                    // output slabs (2: D2H of a chunk overlaps the next chunk's last launch)
     int max_kon_auto = kMaxKon;       // deepest launch the automatic choice considers
+    bool deeper_if_infeasible = false; // ... unless nothing as shallow fits the budget
     bool auto_rounds = false;  // k_off was left to the planner
 
     int64_t interior_planes() const { return n0 - 2 * r; }

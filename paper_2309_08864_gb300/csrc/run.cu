@@ -421,19 +421,23 @@ int plan_create(so2dr_plan_t* out, int ndim, const int64_t* dims, int radius, in
     int rc;
     try {
         P->p.max_kon = maxd;
-        // the automatic choice stays within the register-streaming kernel when
-        // it covers this stencil (the generic kernel is far slower)
-        if (shape == kStar3D && storage != SO2DR_F64 && ndim == 3 && dims && dims[2] % 4 == 0) {
-            int fm = 0;
+        // the automatic choice stays within the streaming kernels' depths (the
+        // generic kernel is far slower: 81-point box FP64 1736x1072, depth 3
+        // 9.4 ms a run, depth 1 4.3; radius 4 star 385x69x90, 16.2 / 2.5).  They
+        // take rows of any length; 16-bit plans, whose results follow the depth,
+        // are bounded only where they always were, on aligned rows of 2D boxes
+        // and 3D stars.  (FP64 in 3D: the plane kernel takes every depth.)
+        const bool exact = storage == SO2DR_F32 || storage == SO2DR_F64;
+        const bool aligned = dims && (ndim == 2 || ndim == 3) && dims[ndim - 1] % 4 == 0;
+        // where a budget leaves room for deeper launches only, those plans stay
+        P->p.deeper_if_infeasible = !(aligned && (shape == kStar3D || shape == kBox2D) && storage != SO2DR_F64);
+        if (ndim == 3 && shape == kStar3D && storage != SO2DR_F64 && (exact || aligned)) {
             for (int d = 1; d <= kMaxKon; ++d)
-                if (fast_star3d_supported(radius, d)) fm = d;
-            if (fm > 0) P->p.max_kon_auto = fm;
+                if (fast_star3d_supported(radius, d)) P->p.max_kon_auto = d;
         }
-        if (shape == kBox2D && storage != SO2DR_F64 && ndim == 2 && dims && dims[1] % 4 == 0) {
-            int fm = 0;
+        if (ndim == 2 && (exact || (shape == kBox2D && aligned))) {
             for (int d = 1; d <= kMaxKon; ++d)
-                if (fast_box2d_supported(radius, d)) fm = d;
-            if (fm > 0) P->p.max_kon_auto = fm;
+                if (row2d_supported(shape, radius, d, csize)) P->p.max_kon_auto = d;
         }
         rc = build_plan(P->p, ndim, dims, radius, kind, coeffs, ncoeffs, time_steps, min_chunks, k_on, k_off,
                         device_budget_bytes, storage, link_h2d_gbs, link_d2h_gbs, hbm_gbs, &err, search);

@@ -6,6 +6,7 @@ import numpy as np
 import pytest
 
 from paper_2309_08864_gb300 import so2dr
+from tests import dispatch
 
 GOLDEN = os.path.join(os.path.dirname(__file__), "golden")
 
@@ -193,3 +194,47 @@ def test_arena_buffers_are_aligned_disjoint_and_inside_the_arena(dims, r, kind, 
             assert a1 <= b0, (mode, (a0, a1), (b0, b1))
         if budget and mode == 0:
             assert arena <= budget
+
+
+@pytest.mark.parametrize("dims,r,kind,dtype,deepest", [
+    ((385, 69, 90), 4, "star", "f32", 2), ((518, 101, 87), 4, "star", "f32", 2), ((91, 171, 81), 4, "star", "f32", 2),
+    ((234, 99, 185), 3, "star", "f32", 2), ((512, 512, 509), 1, "star", "f32", 4), ((778, 918), 3, "box", "f64", 2),
+    ((1736, 1072), 4, "box", "f64", 2), ((802, 1649), 2, "box", "f32", 4), ((700, 701), 1, "star", "f32", 8),
+    ((700, 701), 2, "star", "f64", 4)])
+@pytest.mark.parametrize("k_off", [0, 16])
+def test_automatic_depth_is_one_the_streaming_kernels_take(dims, r, kind, dtype, deepest, k_off):
+    """A depth that only the generic kernel takes is never chosen where a
+    streaming kernel covers the stencil, whatever the row length."""
+    n = (2 * r + 1) ** 2 if kind == "box" else 1 + 2 * len(dims) * r
+    size = 8 if dtype == "f64" else 4
+    for T in (5, 16, 59):
+        for share in (0.3, 0.6):
+            budget = int(size * np.prod(dims) * share) if not k_off else 0
+            p = so2dr.Plan(dims, r, kind, np.full(n, 1.0 / n), T, min_chunks=2, k_off=k_off, budget_bytes=budget, dtype=dtype)
+            k = p.info["k_on"]
+            p.close()
+            assert k <= deepest
+            assert dispatch.launch(dtype, kind, r, k, dims)["fast"] != dispatch.GENERIC
+
+
+def test_budgets_that_fit_deep_launches_only_keep_their_plan():
+    """A round in one launch needs no intermediate slabs: ragged rows, a
+    pinned k_off and a budget that leaves no room for those are still planned,
+    with a depth only the generic kernel takes."""
+    dims, c = (64, 40, 41), np.full(7, 1.0 / 7)
+    deep = so2dr.Plan(dims, 1, "star", c, 20, min_chunks=2, k_on=10, k_off=10, budget_bytes=0, dtype="f32")
+    shallow = so2dr.Plan(dims, 1, "star", c, 20, min_chunks=62, k_on=4, k_off=10, budget_bytes=0, dtype="f32")
+    lo, hi = 0, shallow.info["arena_bytes"]
+    while hi - lo > 1024:  # the least budget any plan of this k_off fits
+        mid = (lo + hi) // 2
+        try:
+            so2dr.Plan(dims, 1, "star", c, 20, min_chunks=2, k_on=10, k_off=10, budget_bytes=mid, dtype="f32").close()
+            hi = mid
+        except so2dr.So2drError:
+            lo = mid
+    with pytest.raises(so2dr.So2drError):
+        so2dr.Plan(dims, 1, "star", c, 20, min_chunks=2, k_on=4, k_off=10, budget_bytes=hi, dtype="f32")
+    p = so2dr.Plan(dims, 1, "star", c, 20, min_chunks=2, k_off=10, budget_bytes=hi, dtype="f32")
+    assert p.info["k_on"] == 10 and p.info["arena_bytes"] <= hi
+    for q in (deep, shallow, p):
+        q.close()
