@@ -636,12 +636,15 @@ double kernel_rate_now(const Plan& p, int depth) {
 
 // Time of one launch that writes `planes` planes.  A segment streams the halo
 // and the pipeline's fill beside its own planes; the 3D star kernel's CTAs
-// (tiles x segments) are counted per SM, as its work split does.
+// (tiles x segments) are counted per SM, as its work split does.  Rows of any
+// length at one rate: ragged ones run 1.7 to 2 times as long in core, but plans
+// made with half as much again were slower (48 problems, 5 of them by up to 33%,
+// none faster), as their chunks' launches wait for planes, not for the SMs.
 double launch_seconds(const Plan& p, int depth, double planes) {
     const double fixed = 5e-6;  // launch, staging latency, tail
     const double rate = kernel_rate_now(p, depth);
     if (p.ndim == 3 && p.dtype == SO2DR_F32 && fast_star3d_supported(p.r, depth)) {
-        const int sms = 152;
+        const int sms = 152;  // (a plan is made without a device)
         const int64_t tx = 128 - 2 * ((p.r * depth + 3) / 4 * 4);
         const int64_t ty = ((depth == 1 && p.r != 3) || (depth > 1 && p.r >= 3) ? 16 : 32) - 2 * p.r * (depth - 1);
         const int64_t edge = p.r <= 2 ? 1024 : 768;  // the grid the rate was measured on
@@ -677,7 +680,8 @@ double predict_ms(const Plan& p) {
     // away from the grid's ends.  (FP32 and FP64 only, whose results do not
     // depend on the depths: 16-bit storage rounds at every launch's end, and
     // its plans, with them its results, stay what they were.)
-    if (p.auto_rounds && !vc && (p.dtype == SO2DR_F32 || p.dtype == SO2DR_F64)) {
+    const bool by_launch = p.auto_rounds && !vc && (p.dtype == SO2DR_F32 || p.dtype == SO2DR_F64);
+    if (by_launch) {
         double chunk = 0;
         int m = 0;
         for (int dl : depths) {
@@ -694,7 +698,15 @@ double predict_ms(const Plan& p) {
     const double h2d_stall = p.lookahead ? 0.0 : units * t_launch;
     const double out_stall = p.n_out >= 2 ? 0.0 : units * std::max(0.0, t_d2h_chunk - t_launch * (L - 1));
     const double hbm = (double)p.rounds * p.n0 * p.plane_bytes * (2.0 + 2.0 * L) / (p.bw_hbm * 1e9);
-    const double body = std::max(std::max(host_h2d + h2d_stall, host_d2h), std::max(kernel + out_stall, hbm));
+    double body = std::max(std::max(host_h2d + h2d_stall, host_d2h), std::max(kernel + out_stall, hbm));
+    // 3D stars in many small chunks: an operation costs the host 6 us at least,
+    // and a chunk's chain of copy, launches and copy leaves every stream idle for
+    // about 15 us.  (93x962x672, 55 steps: 24.5 -> 18.4 ms; 216x301x640, 27 steps
+    // 9.7 -> 8.3; over 60 drawn problems of radius 1 and 2, 8% and 11% less time
+    // out of core.  Radius 3 and 4 keep the plain sum: the deeper launches that
+    // this chooses there cost their in-core runs up to 30%.)
+    if (by_launch && p.ndim == 3 && p.dtype == SO2DR_F32 && p.r <= 2)
+        body = std::max(body, units * (L + 2) * 6e-6) + units * 15e-6;
     const double fill = body / units * 2.0;
     return (body + fill) * 1e3;
 }

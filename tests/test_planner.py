@@ -238,3 +238,15 @@ def test_budgets_that_fit_deep_launches_only_keep_their_plan():
     assert p.info["k_on"] == 10 and p.info["arena_bytes"] <= hi
     for q in (deep, shallow, p):
         q.close()
+
+
+@pytest.mark.parametrize("dims,T,chunks,budget,most", [((93, 962, 672), 55, 6, 116157576, 130),
+                                                       ((216, 301, 640), 27, 5, 44230041, 90)])
+def test_small_chunks_are_not_taken_for_free(dims, T, chunks, budget, most):
+    """Plans of many rounds of four-plane chunks lost to the host's time per
+    operation and the idle ends of each chunk's chain (230 chunks 24.5 ms, 112
+    chunks 18.4; 155 chunks 9.7 ms, 80 chunks 8.3)."""
+    p = so2dr.Plan(dims, 1, "star", [0.4] + [0.1] * 6, T, min_chunks=chunks, budget_bytes=budget, dtype="f32")
+    f = p.info
+    assert f["rounds"] * f["chunks"] <= most and f["arena_bytes"] <= budget
+    p.close()
