@@ -89,7 +89,10 @@ template <int R, int K, bool SMALL = false> struct StarShape {
     // 461 at one level, 110 / 245 at two, radius 3 485 / 515 and 329 / 357,
     // 1024^3 radius 2 770 / 859 at two)
     static constexpr int UNR = R == 1 && !SMALL ? 2 : 1;
-    static constexpr int MINB = SMALL || (K == 1 && R != 3) ? 2 : 1;         // CTAs per SM the registers are sized for
+    // CTAs per SM the registers are sized for.  Radius 2 at one level: three
+    // (80 registers; at two it takes 106: 20x400x1000 27.1 -> 20.7 us a launch,
+    // 459x300x728 187 -> 170, 512^3 215 -> 205, 256^3 62 -> 65)
+    static constexpr int MINB = R == 2 && K == 1 ? 3 : SMALL || (K == 1 && R != 3) ? 2 : 1;
     // staged columns: 16-bit boxes start on an 8-element boundary (16 bytes),
     // so they carry 8 spare columns and the tile starts 0 or 4 columns in
     template <int ES> static constexpr int lxb() { return ES == 4 ? LX : LX + 8; }
@@ -761,7 +764,7 @@ struct StarTB {
 // One instantiation per staging mode, so that the launches of the copy-engine
 // pipeline on aligned rows carry none of the others' code
 template <typename T, int R, int K, int STG = kStageTma, bool SMALL = false>
-__global__ void __launch_bounds__(StarShape<R, K>::NT, STG == kStageRagged && (R > 2 || SMALL) ? 1 : StarShape<R, K, SMALL>::MINB)
+__global__ void __launch_bounds__(StarShape<R, K>::NT, STG == kStageRagged && (R > 2 || SMALL) ? 1 : STG == kStageRagged && R == 2 && K == 1 ? 2 : StarShape<R, K, SMALL>::MINB)
     star3d_tb_kernel(const StencilArgs a, const __grid_constant__ CUtensorMap tmap) {
     extern __shared__ __align__(1024) unsigned char smem_tb[];
     StarTB<T, R, K, STG, SMALL> k(a, &tmap);

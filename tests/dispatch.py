@@ -32,3 +32,9 @@ def launch(dtype, kind, r, depth, dims, nout=None, sms=152, occ=4):
     _lib().probe_launch(so2dr.DTYPES[dtype], SHAPES[kind, len(dims)], r, depth, i64(n0), i64(ny), i64(nx),
                         i64(nout or n0), sms, occ, out)
     return dict(zip(FIELDS, out))
+
+
+def star_occupancy(dtype, r, depth, dims):
+    """CTAs per SM of the 3D star kernel (needs a GPU)."""
+    i64 = ctypes.c_int64
+    return _lib().probe_star_occupancy(so2dr.DTYPES[dtype], r, depth, *(i64(n) for n in dims))

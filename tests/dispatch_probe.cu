@@ -25,3 +25,11 @@ extern "C" void probe_launch(int dtype, int shape, int r, int depth, int64_t n0,
                            a.split, a.split2, a.split_at};
     for (int i = 0; i < 13; ++i) out[i] = v[i];
 }
+
+// CTAs per SM the driver reports for the 3D star kernel of a launch (needs a
+// GPU); -1: another kernel.
+extern "C" int probe_star_occupancy(int dtype, int r, int depth, int64_t n0, int64_t ny, int64_t nx) {
+    const int esize = dtype == SO2DR_F32 ? 4 : 2;
+    LaunchShape ls = stencil_launch_shape(kStar3D, r, depth, n0, ny, nx, 4, esize);
+    return ls.ok && ls.fast == kFastStar3D ? stencil_occupancy(dtype, kStar3D, r, depth, ls) : -1;
+}
