@@ -404,8 +404,19 @@ void choose_row_split(LaunchShape& ls, int64_t nout, int r, int depth, int csize
             if (n < 1) n = 1;
             if (n > nout) n = nout;
             const int64_t per_sm = (strips * n * slots + G - 1) / G;
-            const int64_t busy = per_sm <= slots ? (per_sm > wmin ? per_sm : wmin) : (per_sm + slots - 1) / slots * slots;
-            const double cost = (double)busy * ((double)((nout + n - 1) / n) + ovh);
+            int64_t busy = per_sm <= slots ? (per_sm > wmin ? per_sm : wmin) : (per_sm + slots - 1) / slots * slots;
+            double uneven = 1.0;
+            if (csize == 8 && per_sm <= slots) {
+                // FP64: a CTA's warps fill an SM, so whole CTAs per SM count; and
+                // with fewer than the SMs hold evenly, some get one more all the
+                // same (134 to 138 CTAs took 1.4 times as long a row as 144 to 149).
+                // Us a launch with fewer / even CTAs: 9-point box, four levels,
+                // 600x12800 847 / 572, radius 1 star 484 / 321
+                const int64_t ctas = (strips * n + kRowWarps - 1) / kRowWarps, lev = (ctas + sms - 1) / sms;
+                busy = kRowWarps * lev;
+                if (ctas < 0.93 * lev * sms) uneven = 1.0 + 0.4 / lev;
+            }
+            const double cost = (double)busy * ((double)((nout + n - 1) / n) + ovh) * uneven;
             if (best < 0 || cost < best * 0.98) { a.split = (int)n; best = cost; }
         }
     }
@@ -416,21 +427,21 @@ bool tile2d_short(LaunchShape& ls, int shape, int64_t nout, int64_t nx, int r, i
     // Rows of 32 columns per SM up to which the tile is the faster one
     // (in-core Gcell-steps/s, strips / tile).  FP64, fused: 80x512 radius 1, 4
     // levels 5.6 / 15.7, 512^2 28 / 43, 1024^2 60 / 73 (215 rows per SM).
-    // FP64, wide halos: a segment streams more halo than rows of its own (us a
-    // launch, strips / tile / generic kernel).  One level, radius 2 star
-    // 64x1000 14.5 / 8.7 / 13.4, 300x12800 (789 rows) 133 / 77 / 146; 25-point
-    // box 250x6000 102 / 104 / 142, 300x12800 357 / 226 / 281; radius 4 star
-    // 75x3882 43 / 21 / 35, 300x12800 264 / 133 / 207; 81-point box 250x6000
-    // 357 / 293 / 314, 2000^2 (829 rows) 807 / 698 / 910.  Two levels, 81-point
-    // box 500x6000 (618 rows) 1255 / 1155 / 1233, 2000^2 1578 / 1623 / 1798;
-    // 49-point box 1000x3882 (802 rows) 872 / 946 / 1072.  Radius 1 at one
-    // level has little halo to save (512^2 20.9 / 20.3 Gcell-steps/s).  FP32: 81-point box,
+    // FP64, one level: the tile at any size (us a launch, strips / tile /
+    // generic kernel: radius 1 star 4096^2 210 / 174 / 490, 9-point box 300x12800
+    // 127 / 76 / 111, radius 4 star 75x3882 43 / 21 / 35, 8000x8192 2580 / 2130 /
+    // 2659, 81-point box 4096^2 3681 / 2758 / 3200), but the 25-point box up to
+    // 1024 rows (300x12800 357 / 226 / 281; 2001x5003 579 / 612 / 646).  FP64, two
+    // levels of radius 3 and 4: 81-point box 500x6000 (618 rows) 1255 / 1155 /
+    // 1233, 2000^2 1578 / 1623 / 1798; 49-point box 1000x3882 (802 rows) 872 /
+    // 946 / 1072; ragged rows 81-point box 2001x5003 (2067 rows) 4613 / 3959 /
+    // 4104, radius 3 star 763 / 601 / 1209.  FP32: 81-point box,
     // one level 512^2 14.0 / 18.8, 1024^2 49 / 52; radius 3, 4 levels,
     // 701x1003 93 / 106; 9-point box, 8 levels 512^2 74 / 85 (54 rows), 1024^2
     // 272 / 219; radius 1, 4 levels 80x512 18 / 20, 256^2 (13 rows) 26 / 25,
     // 512^2 94 / 72.
     const int H = r * depth;
-    const int64_t limit = csize == 8 ? (depth == 1 ? (r > 1 ? 1024 : 0) : r > 2 ? 640 : 256)
+    const int64_t limit = csize == 8 ? (depth == 1 ? (shape == kBox2D && r == 2 ? 1024 : 1 << 30) : r > 2 ? (ls.ragged ? 2200 : 640) : 256)
                           : (shape == kBox2D && r >= 3) || H >= 12 ? 160
                           : H >= 6 ? 60 : depth > 1 ? 12 : 0;
     const int64_t gx = (nx + kTileX - 1) / kTileX;

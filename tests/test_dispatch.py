@@ -46,14 +46,17 @@ def test_zero_copy_only_where_the_star_kernel_runs(dtype, r, k):
     assert zc(64, 40, 24)[0] and not zc(64, rows + 1, 24)[0] and not zc(64, 9, (1 << 30) + 8)[0]
 
 
-@pytest.mark.parametrize("kind,r,k", [(kind, r, 1) for kind in ("star", "box") for r in (2, 3, 4)] + [("box", 4, 2), ("star", 3, 2)])
+@pytest.mark.parametrize("kind,r,k", [(kind, r, 1) for kind in ("star", "box") for r in (1, 2, 3, 4)] + [("box", 4, 2), ("star", 3, 2)])
 def test_short_fp64_launches_take_the_tile(kind, r, k):
     """Chunk launches of wide halos in FP64: the strips' segments stream
     mostly halo there and were slower than the generic kernel."""
     for dims, nout in [((599, 3882), 75), ((140, 2112), 140), ((64, 1000), 64), ((20, 3882), 20), ((250, 6000), 250),
                        ((12800, 12800), 300 if k == 1 else 200)]:
         assert dispatch.launch("f64", kind, r, k, dims, nout)["fast"] == dispatch.TILE2D
-    assert dispatch.launch("f64", kind, r, k, (12800, 12800))["fast"] == dispatch.ROW2D
+    if r >= 3 and k == 2:  # ragged rows, staged element by element
+        assert dispatch.launch("f64", kind, r, k, (2001, 5003))["fast"] == dispatch.TILE2D
+    large = dispatch.launch("f64", kind, r, k, (12800, 12800))
+    assert large["fast"] == (dispatch.TILE2D if k == 1 and (kind, r) != ("box", 2) else dispatch.ROW2D)
 
 
 @pytest.mark.parametrize("dims,r,k,small", [
@@ -82,3 +85,11 @@ def test_small_fp64_plane_launches_fill_the_device(kind, r, k, dims):
     assert sh["gx"] * sh["tx"] >= dims[2] and sh["gy"] * sh["ty"] >= dims[1] and sh["smem"] <= 227 << 10
     assert 1 <= sh["gz"] <= dims[0]
     assert dispatch.launch("f32", "varcoef", 1, 2, dims)["tx"] == dispatch.launch("f32", "varcoef", 1, 2, (4000,) + dims[1:])["tx"]
+
+
+@pytest.mark.parametrize("kind,r,k,dims", [("box", 1, 4, (600, 12800)), ("box", 2, 1, (1000, 8192)), ("star", 1, 4, (600, 12800)),
+                                           ("star", 2, 2, (1000, 8192)), ("box", 1, 2, (1000, 8192))])
+def test_fp64_strips_are_split_into_ctas_that_share_the_sms_evenly(kind, r, k, dims):
+    """A few CTAs less than the SMs hold evenly double up on some of them."""
+    sh = dispatch.launch("f64", kind, r, k, dims, occ=3)
+    assert sh["fast"] == dispatch.ROW2D and sh["gx"] >= 0.93 * 152 * -(-sh["gx"] // 152)

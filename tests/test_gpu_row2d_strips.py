@@ -19,7 +19,7 @@ BOX = [(1, k) for k in range(1, 9)] + [(2, 1), (2, 2), (2, 3), (2, 4), (3, 1), (
 STAR = [(1, k) for k in range(1, 9)] + [(r, k) for r in (2, 3, 4) for k in (1, 2, 3, 4)]
 WIDE = [(1, 1), (1, 2), (1, 3), (1, 4), (2, 1), (2, 2), (2, 3), (2, 4), (3, 1), (3, 2), (4, 1), (4, 2)]  # FP64
 CASES = [("box", r, k, "f32") for r, k in BOX] + [("star", r, k, "f32") for r, k in STAR]
-CASES += [(kind, r, k, "f64") for kind in ("box", "star") for r, k in WIDE]
+CASES += [(kind, r, k, "f64") for kind in ("box", "star") for r, k in WIDE if k > 1 or (kind, r) == ("box", 2)]
 CASES += [("box", 1, 8, "bf16"), ("box", 3, 2, "bf16"), ("box", 4, 1, "f16"), ("star", 2, 4, "f16"),
           ("star", 1, 4, "bf16"), ("star", 4, 3, "bf16")]
 
@@ -57,6 +57,8 @@ def _same_bytes(dims, kind, r, k, name, modes, monkeypatch):
                                   (17, 294000), (17, 294001)])
 @pytest.mark.parametrize("kind,r,k,name", CASES)
 def test_strips_match_generic_kernel_bitwise(kind, r, k, name, dims, monkeypatch):
+    if name == "f64" and r > 2 and dims[1] % 4:  # the tile takes these up to twice as many rows
+        dims = (dims[0] * 9 // 4, dims[1])
     sh = dispatch.launch(name, kind, r, k, dims, sms=_sms())
     wide = kind == "box" and (r, k) == (2, 4) and name != "f64" and dims[1] % 4 == 0
     assert sh["fast"] == (dispatch.BOX2D if wide else dispatch.ROW2D)
@@ -67,7 +69,7 @@ def test_strips_match_generic_kernel_bitwise(kind, r, k, name, dims, monkeypatch
 @pytest.mark.parametrize("kind,r,k,name", [("box", 1, 8, "f32"), ("box", 1, 1, "f32"), ("box", 4, 2, "f32"),
                                            ("box", 2, 3, "bf16"), ("box", 2, 2, "f64"), ("star", 1, 8, "f32"),
                                            ("star", 3, 4, "f32"), ("star", 1, 4, "f16"), ("star", 2, 4, "f64"),
-                                           ("star", 4, 1, "f64")])
+                                           ("star", 4, 2, "f64")])
 def test_long_and_short_segments_match_generic_kernel_bitwise(kind, r, k, name, dims, monkeypatch):
     for occ in range(1, 5):  # whatever number of CTAs fits an SM
         sh = dispatch.launch(name, kind, r, k, dims, sms=_sms(), occ=occ)
@@ -75,8 +77,8 @@ def test_long_and_short_segments_match_generic_kernel_bitwise(kind, r, k, name, 
     _same_bytes(dims, kind, r, k, name, (1, 0), monkeypatch)
 
 
-@pytest.mark.parametrize("dims", [(75, 3882), (64, 1000), (33, 125), (20, 31)])
-@pytest.mark.parametrize("kind,r,k", [(kind, r, 1) for kind in ("star", "box") for r in (2, 3, 4)] + [("box", 4, 2), ("star", 3, 2)])
-def test_fp64_tile_of_wide_halos_matches_generic_kernel_bitwise(kind, r, k, dims, monkeypatch):
+@pytest.mark.parametrize("dims", [(75, 3882), (64, 1000), (33, 125), (20, 31), (900, 5003)])
+@pytest.mark.parametrize("kind,r,k", [(kind, r, 1) for kind in ("star", "box") for r in (1, 2, 3, 4)] + [("box", 4, 2), ("star", 3, 2)])
+def test_fp64_tile_matches_generic_kernel_bitwise(kind, r, k, dims, monkeypatch):
     assert dispatch.launch("f64", kind, r, k, dims, sms=_sms())["fast"] == dispatch.TILE2D
     _same_bytes(dims, kind, r, k, "f64", (1, 0), monkeypatch)
