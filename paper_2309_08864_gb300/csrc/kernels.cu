@@ -39,10 +39,10 @@ bool fast_box2d_supported(int r, int depth) {
 
 // Radius 2, four levels, on 12800^2 FP32: 825 Gcell-steps/s against 730 with
 // the warp strips of row2d_tb.cuh, which give 16 of their 128 columns to the
-// halo there; every other (R, K) is faster in strips (radius 1: 1763 / 1504 at
+// halo there.  The other (R, K) are faster in strips (radius 1: 1763 / 1504 at
 // 8 levels, 1828 / 1289 at 4; radius 2: 730 / 605 at 1, 759 / 670 at 2;
-// radius 3: 481 / 368 at 1, 403 / 404 at 3; radius 4: 321 / 246 at 1,
-// 287 / 239 at 2).
+// radius 3: 481 / 368 at 1; radius 4: 321 / 246 at 1, 287 / 239 at 2), or the
+// same (radius 3 at 3 levels: 403 / 404).
 bool wide_box2d(int r, int depth, int64_t nx, int csize) { return r == 2 && depth == 4 && nx % 4 == 0 && csize == 4; }
 
 bool row2d_supported(int shape, int r, int depth, int csize) {

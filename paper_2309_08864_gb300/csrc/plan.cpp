@@ -564,13 +564,13 @@ void trapezoid_work(const Plan& p, double* computed, double* useful) {
     *useful = u;
 }
 
-// Measured in-core rates (cell updates per second, in-plane halo work
-// included) of the kernels on one GB300: the register-streaming 3D star kernel
-// by radius and depth, and the generic kernel.
+// In-core rates (cell updates per second, in-plane halo work included) by which
+// 16-bit storage, variable coefficients and plans of a given k_off are made.
+// They are those of earlier kernels and stay as they are: a 16-bit plan's depths
+// decide where its results are rounded.  (kernel_rate_now has the present ones.)
 double kernel_rate(const Plan& p, int depth) {
     if (p.kind == SO2DR_BOX && p.ndim == 2 && p.dtype != SO2DR_F64 && p.nx % 4 == 0 && depth <= p.max_kon_auto) {
-        // 2D box kernel, in-core cell-steps/s measured on 16384^2 FP32
-        // (unmeasured depths interpolated)
+        // CTA-wide 2D box kernel, 16384^2 FP32 (unmeasured depths interpolated)
         static const double b1[9] = {0, 757e9, 1029e9, 1120e9, 1203e9, 1250e9, 1300e9, 1340e9, 1368e9};
         static const double b2[5] = {0, 557e9, 703e9, 745e9, 786e9};
         static const double b3[4] = {0, 371e9, 375e9, 384e9};
@@ -585,8 +585,7 @@ double kernel_rate(const Plan& p, int depth) {
     bool fast = p.kind == SO2DR_STAR && p.ndim == 3 && p.dtype != SO2DR_F64 && p.nx % 4 == 0 &&
                 depth <= p.max_kon_auto;
     if (!fast) return p.dtype == SO2DR_F64 ? 20e9 : 100e9;
-    // (in-core, 1024^3 FP32; radius 3 and 4 at depth 2 run 2 rows per warp
-    // and 2R = 6 or 8 unrolled phases, far slower than one level)
+    // (1024^3 FP32)
     if (p.r == 1) {
         const double r1[5] = {0, 815e9, 1280e9, 1470e9, 1510e9};
         return r1[std::min(depth, 4)];

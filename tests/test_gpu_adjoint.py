@@ -55,6 +55,26 @@ def test_adjoint_matches_oracle(dtype, dims, T, C, budget, K, monkeypatch):
     plan.close()
 
 
+@pytest.mark.parametrize("dtype", [so2dr.F64, so2dr.F32])
+@pytest.mark.parametrize("dims", [(9, 19, 71), (14, 9, 33), (40, 25, 64)])
+def test_adjoint_of_several_blocks_matches_oracle(dims, dtype):
+    """Grids of more than one block of columns (32 x 8) each way, with partial
+    ones, and planes split over several blocks."""
+    import torch
+    T, C = 6, 3
+    u0, faces, tgt, tu0, tf, tt = _problem(dims, dtype)
+    plan = so2dr.Plan(dims, 1, "varcoef", None, T, min_chunks=2, k_on=2, k_off=C, budget_bytes=0, dtype=dtype)
+    gu_, gc_ = torch.empty_like(tu0).pin_memory(), torch.empty_like(tf).pin_memory()
+    loss, _ = plan.adjoint(tu0, tf, tt, gu_, gc_, plan.workspace(C), C)
+    L, gref_u, gref_c = oracle.adjoint_varcoef(u0.astype(np.float64), faces.astype(np.float64),
+                                               tgt.astype(np.float64), T, ckpt_every=C)
+    tol = 1e-12 if dtype == so2dr.F64 else 2e-5  # the tolerances of the small grids above
+    assert abs(loss - L) <= tol * abs(L) * 10
+    assert gu.rel_linf(gu_.numpy().astype(np.float64), gref_u) <= tol
+    assert gu.rel_linf(gc_.numpy().astype(np.float64), gref_c) <= tol
+    plan.close()
+
+
 def test_dot_is_fp64_exact_enough():
     import torch
     n = 3_000_001
