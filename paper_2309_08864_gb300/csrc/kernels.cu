@@ -309,6 +309,9 @@ void choose_work_split(LaunchShape& ls, int64_t nout, int r, int depth, int sms,
     } else {
         ls.grid.z = (unsigned)nseg;
     }
+    // radius 2 at one level: registers for two CTAs per SM, not three, where
+    // the launch has no more (star3d_tb.cuh)
+    ls.small = r == 2 && depth == 1 && !ls.ragged && (int64_t)ls.grid.x * ls.grid.y * ls.grid.z <= 2 * (int64_t)sms;
 }
 
 // FP64 launches of up to this many cells get a tile of their own.  Us a launch,

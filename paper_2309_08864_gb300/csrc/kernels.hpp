@@ -17,7 +17,7 @@ struct LaunchShape {
     bool ok;
     int fast;    // 0 generic kernel, kFastStar3D (star3d_tb.cuh), kFastRow2D (row2d_tb.cuh),
                  // kFastBox2D (box2d_fast.cuh), kFastPlane3D (plane_tb.cuh), kFastTile2D (tile2d_tb.cuh)
-    bool small;  // 3D star kernel: the 2-row tile (star_small)
+    bool small;  // 3D star kernel: its form for few CTAs (star_small, choose_work_split)
     bool ragged; // rows are not whole 4-element vectors: the kernels' element-wise staging
 };
 

@@ -248,6 +248,7 @@ int enqueue_stencil(so2dr_plan_s* P, const RunList& rl, const Op& op, cudaStream
             // (the grid is chosen with the tile)
         } else if (ls.fast == kFastStar3D) {
             choose_work_split(ls, o.dst_hi - o.dst_lo, p.r, o.depth, P->sm_count, occ, &a.split);
+            if (op.host_src >= 0) ls.small = false;  // (the host-reading form is built for three)
             // the round split's piece counter: one per stream (the launches
             // of a stream run one after another), beside the status word
             if (a.split && o.stream >= 0 && o.stream < kNumStreams)

@@ -63,9 +63,10 @@ namespace so2dr {
 // Gcell-steps/s; radius 2 loses, 702 -> 626, radius 4 is the same).
 // SMALL (radius 1 fused, radius 3 at one level): 2 rows per warp and two CTAs
 // per SM, for grids of so few tiles that a CTA's own pace counts
-// (star_small in kernels.cu).
+// (star_small in kernels.cu); radius 2 at one level: the same tile with
+// registers for two CTAs (choose_work_split).
 template <int R, int K, bool SMALL = false> struct StarShape {
-    static constexpr bool HAS_SMALL = (R == 1 && K > 1) || (R == 3 && K == 1);
+    static constexpr bool HAS_SMALL = (R == 1 && K > 1) || ((R == 2 || R == 3) && K == 1);
     static constexpr int VY = SMALL ? 2 : R == 3 && K == 1 ? 4 : (K == 1 || R >= 3) ? 2 : 4;
     static constexpr int NW = 8;
     static constexpr int NT = NW * 32;
@@ -91,8 +92,10 @@ template <int R, int K, bool SMALL = false> struct StarShape {
     static constexpr int UNR = R == 1 && !SMALL ? 2 : 1;
     // CTAs per SM the registers are sized for.  Radius 2 at one level: three
     // (80 registers; at two it takes 106: 20x400x1000 27.1 -> 20.7 us a launch,
-    // 459x300x728 187 -> 170, 512^3 215 -> 205, 256^3 62 -> 65)
-    static constexpr int MINB = R == 2 && K == 1 ? 3 : SMALL || (K == 1 && R != 3) ? 2 : 1;
+    // 459x300x728 187 -> 170, 512^3 215 -> 205), and two where a launch has no
+    // more CTAs than that, which gains nothing from the third (SMALL: 256^3 65 ->
+    // 62, BF16 194x164x16 18.0 -> 16.4)
+    static constexpr int MINB = R == 2 && K == 1 && !SMALL ? 3 : SMALL || (K == 1 && R != 3) ? 2 : 1;
     // staged columns: 16-bit boxes start on an 8-element boundary (16 bytes),
     // so they carry 8 spare columns and the tile starts 0 or 4 columns in
     template <int ES> static constexpr int lxb() { return ES == 4 ? LX : LX + 8; }

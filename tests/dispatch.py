@@ -34,6 +34,11 @@ def launch(dtype, kind, r, depth, dims, nout=None, sms=152, occ=4):
     return dict(zip(FIELDS, out))
 
 
+def star_split_small(dtype, r, depth, dims, sms=152, occ=3):
+    i64 = ctypes.c_int64
+    return _lib().probe_star_split_small(so2dr.DTYPES[dtype], r, depth, *(i64(n) for n in dims), sms, occ)
+
+
 def star_occupancy(dtype, r, depth, dims):
     """CTAs per SM of the 3D star kernel (needs a GPU)."""
     i64 = ctypes.c_int64

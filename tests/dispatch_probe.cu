@@ -26,6 +26,15 @@ extern "C" void probe_launch(int dtype, int shape, int r, int depth, int64_t n0,
     for (int i = 0; i < 13; ++i) out[i] = v[i];
 }
 
+// Whether a 3D star launch's split takes the form for few CTAs.
+extern "C" int probe_star_split_small(int dtype, int r, int depth, int64_t n0, int64_t ny, int64_t nx, int sms, int occ) {
+    LaunchShape ls = stencil_launch_shape(kStar3D, r, depth, n0, ny, nx, 4, dtype == SO2DR_F32 ? 4 : 2);
+    ls.grid.z = 1;
+    int split = 0;
+    choose_work_split(ls, n0, r, depth, sms, occ, &split);
+    return ls.small;
+}
+
 // CTAs per SM the driver reports for the 3D star kernel of a launch (needs a
 // GPU); -1: another kernel.
 extern "C" int probe_star_occupancy(int dtype, int r, int depth, int64_t n0, int64_t ny, int64_t nx) {

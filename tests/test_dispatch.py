@@ -93,3 +93,12 @@ def test_fp64_strips_are_split_into_ctas_that_share_the_sms_evenly(kind, r, k, d
     """A few CTAs less than the SMs hold evenly double up on some of them."""
     sh = dispatch.launch("f64", kind, r, k, dims, occ=3)
     assert sh["fast"] == dispatch.ROW2D and sh["gx"] >= 0.93 * 152 * -(-sh["gx"] // 152)
+
+
+def test_radius_two_registers_follow_the_ctas_of_the_launch():
+    """One level of radius 2: registers for three CTAs per SM only where the
+    launch has more than two."""
+    for dims, small in [((256, 256, 256), 1), ((194, 164, 16), 1), ((20, 400, 1000), 0), ((459, 300, 728), 0), ((256, 256, 255), 0)]:
+        assert dispatch.star_split_small("f32", 2, 1, dims) == small, dims
+    for r, k in RK:
+        assert (r, k) == (2, 1) or dispatch.star_split_small("f32", r, k, (256, 256, 256)) == 0
